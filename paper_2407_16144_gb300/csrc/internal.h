@@ -167,7 +167,7 @@ int row_iter_blocks_per_sm(int smem, int threads);
 // ---- standalone KKT evaluation (kkt.cu) --------------------------------------------------------
 constexpr int kKktMaxBlocks = 1024;   // block partials of the evaluation kernels
 constexpr int kKktSlotCount = 8;
-int kkt_blocks(int m, int n);
+int kkt_blocks(int rows);
 // scratch: kty (n doubles), part (kKktMaxBlocks * kKktSlotCount doubles), dout (8 doubles);
 // *bad_index is set when the CSR held a row offset or column index out of range
 cudaError_t kkt_eval_with_scratch(const rhpdhg_problem *lp, const double *x, const double *y,

@@ -11,10 +11,12 @@
 // partials and finished by one block.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 #include <string>
 
 #include "../../include/rhpdhg.h"
+#include "bufcache.h"
 #include "internal.h"
 
 namespace rh {
@@ -24,7 +26,11 @@ namespace {
 constexpr int kKktThreads = 256;
 constexpr int kKktSlots = kKktSlotCount;   // stride of a block's partials
 constexpr int kKktUsed = 7;                // 0 rp2, 1 qy, 2 qq, 3 rd2, 4 cx, 5 bnd, 6 cc
+constexpr int kKktRowSlots = 3;            // the first three come from the row kernel
 constexpr int kKktFlag = 5;                // dout[5]: 1 if the CSR held an index out of range
+constexpr int kKktStage = 704;             // entries a warp stages at a time (22 per row of 32)
+constexpr int kKktUnroll = 4;              // entries per lane in flight
+constexpr int kKktRowCtas = 4;             // resident CTAs per SM of the row kernel (45 KB each)
 
 __device__ __forceinline__ double block_sum(double v, double *sh) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -38,37 +44,97 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
   return r;   // valid in thread 0
 }
 
+// One warp takes 32 consecutive rows: their entries are read as one contiguous segment, kKktStage at
+// a time, every lane on consecutive entries (one thread per row read 12 bytes here and 12 bytes
+// 200 bytes further on).  Each entry finds its row among the 32 row ends by a search in shuffles,
+// scatters val * y_row and stages val * x_j in shared memory, from which the rows are summed
+// balanced over the lanes (balanced_row_sum).  Bound by the FP64 pipe (62% busy; two products and
+// one sum per entry) and the scattered FP64 additions in L2: 280 us for 30M entries.  The whole
+// evaluation of that LP took 950 us with a thread per row, a cudaMalloc and cudaFree per call and
+// floating-point comparisons in the column kernel, and takes 464 us.
+//
 // Rows whose offsets fall outside [0, nnz] or decrease, and entries whose column lies outside
-// [0, n), are skipped and reported through flag (the caller's CSR is not validated beforehand).
-__global__ void __launch_bounds__(kKktThreads)
-k_kkt_rows(int m, int m_eq, int n, long long nnz, const long long *rp, const int *col,
-           const double *val, const double *x, const double *y, const double *q, double *kty,
-           double *part, double *flag) {
+// [0, n), are skipped and reported through flag (the caller's CSR is not validated beforehand);
+// 32 rows with such an offset among them are walked one thread per row.
+__global__ void __launch_bounds__(kKktThreads, kKktRowCtas)
+k_kkt_rows(int m, int m_eq, int n, long long nnz, const long long *__restrict__ rp,
+           const int *__restrict__ col, const double *__restrict__ val,
+           const double *__restrict__ x, const double *__restrict__ y,
+           const double *__restrict__ q, double *kty, double *part, double *flag) {
   __shared__ double sh[kKktThreads / 32];
+  __shared__ double staged[kKktThreads / 32][kKktStage];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  double *st = staged[threadIdx.x >> 5];
   double s_rp2 = 0.0, s_qy = 0.0, s_qq = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < m;
-       i += (long long)gridDim.x * blockDim.x) {
-    const double yi = y[i], qi = q[i];
+  const long long nwarps = (long long)gridDim.x * (kKktThreads / 32);
+  for (long long t = blockIdx.x * (kKktThreads / 32) + (threadIdx.x >> 5); t * 32 < m;
+       t += nwarps) {
+    const long long i = t * 32 + lane;
+    const bool in = i < m;
+    const long long p0 = rp[in ? i : m], p1 = rp[in ? i + 1 : m];
+    const double yi = in ? y[i] : 0.0, qi = in ? q[i] : 0.0;
     double kx = 0.0;
-    long long p0 = rp[i], p1 = rp[i + 1];
-    if (p0 < 0 || p1 < p0 || p1 > nnz) {
-      *flag = 1.0;
-      p1 = p0;
-    }
-    for (long long p = p0; p < p1; ++p) {
-      const int j = col[p];
-      if (j < 0 || j >= n) {
-        *flag = 1.0;
-        continue;
+    const bool bad = p0 < 0 || p1 < p0 || p1 > nnz;
+    if (__any_sync(full, bad)) {
+      if (bad && in) *flag = 1.0;
+      for (long long p = p0; in && !bad && p < p1; ++p) {
+        const int j = col[p];
+        if (j < 0 || j >= n) {
+          *flag = 1.0;
+          continue;
+        }
+        kx += val[p] * x[j];
+        atomicAdd(kty + j, val[p] * yi);
       }
-      kx += val[p] * x[j];
-      atomicAdd(kty + j, val[p] * yi);
+    } else {
+      const long long seg_e = __shfl_sync(full, p1, 31);
+      for (long long base = __shfl_sync(full, p0, 0); base < seg_e; base += kKktStage) {
+        const int len = (int)min((long long)kKktStage, seg_e - base);
+        const int lo = (int)min(max(p0 - base, 0ll), (long long)len);
+        const int hi = (int)min(max(p1 - base, 0ll), (long long)len);
+        for (int o = 0; o < len; o += 32 * kKktUnroll) {
+          int j[kKktUnroll];
+          double v[kKktUnroll], xj[kKktUnroll];
+#pragma unroll
+          for (int u = 0; u < kKktUnroll; ++u) {
+            const int k = o + 32 * u + lane;
+            j[u] = k < len ? col[base + k] : 0;
+            v[u] = k < len ? val[base + k] : 0.0;
+          }
+#pragma unroll
+          for (int u = 0; u < kKktUnroll; ++u) {
+            const bool ok = j[u] >= 0 && j[u] < n;
+            if (!ok) *flag = 1.0;
+            xj[u] = ok && o + 32 * u + lane < len ? x[j[u]] : 0.0;
+          }
+#pragma unroll
+          for (int u = 0; u < kKktUnroll; ++u) {
+            const int k = o + 32 * u + lane;
+            int r = 0;                       // rows that end at or before entry k
+#pragma unroll
+            for (int h = 16; h > 0; h >>= 1)
+              if (__shfl_sync(full, hi, r + h - 1) <= k) r += h;
+            const double yr = __shfl_sync(full, yi, r);
+            if (k < len) {
+              const bool ok = j[u] >= 0 && j[u] < n;
+              st[k] = ok ? v[u] * xj[u] : 0.0;
+              if (ok) atomicAdd(kty + j[u], v[u] * yr);
+            }
+          }
+        }
+        __syncwarp();
+        kx += balanced_row_sum(st, len, lo, hi);
+        __syncwarp();
+      }
     }
-    double r = qi - kx;
-    if (i >= m_eq) r = fmax(r, 0.0);
-    s_rp2 += r * r;
-    s_qy += qi * yi;
-    s_qq += qi * qi;
+    if (in) {
+      double r = qi - kx;
+      if (i >= m_eq) r = fmax(r, 0.0);
+      s_rp2 += r * r;
+      s_qy += qi * yi;
+      s_qq += qi * qi;
+    }
   }
   const double a = block_sum(s_rp2, sh), b = block_sum(s_qy, sh), c = block_sum(s_qq, sh);
   if (threadIdx.x == 0) {
@@ -87,16 +153,19 @@ k_kkt_cols(int n, const double *c, const double *l, const double *u, const doubl
        j += (long long)gridDim.x * blockDim.x) {
     const double cj = c[j], lj = l[j], uj = u[j];
     const double g = cj - kty[j];
-    const bool lf = isfinite(lj), uf = isfinite(uj);
+    // The FP64 pipe bounds this kernel: six FP64 instructions per column are left, with the
+    // comparisons on the integer pipe (10M columns: 291 us with floating-point comparisons, 80% of
+    // the pipe, about 130 us without).
+    const bool lf = dbl_finite(lj), uf = dbl_finite(uj);
     double lam = 0.0;
     if (lf && uf) lam = g;
-    else if (lf) lam = fmax(g, 0.0);
-    else if (uf) lam = fmin(g, 0.0);
+    else if (lf) lam = dbl_pos(g) ? g : 0.0;
+    else if (uf) lam = dbl_neg(g) ? g : 0.0;
     const double rd = g - lam;
     s_rd2 += rd * rd;
     s_cx += cj * x[j];
-    if (lam > 0.0) s_bnd += lj * lam;
-    else if (lam < 0.0) s_bnd += uj * lam;
+    const bool pos = dbl_pos(lam), neg = dbl_neg(lam);
+    s_bnd += (pos ? lj : neg ? uj : 0.0) * (pos || neg ? lam : 0.0);
     s_cc += cj * cj;
   }
   const double a = block_sum(s_rd2, sh), b = block_sum(s_cx, sh), d = block_sum(s_bnd, sh),
@@ -109,14 +178,18 @@ k_kkt_cols(int n, const double *c, const double *l, const double *u, const doubl
   }
 }
 
-__global__ void k_kkt_final(int nb, const double *part, double off, double *out) {
-  // one thread per used slot, blocks summed in order
+// One warp per used slot: lane l adds blocks l, l + 32, ... in order, then a fixed shuffle tree (one
+// thread per slot spent about 1000 dependent FP64 additions on a full grid).
+__global__ void __launch_bounds__(32 * kKktUsed)
+k_kkt_final(int nb_rows, int nb_cols, const double *part, double off, double *out) {
   __shared__ double tot[kKktUsed];
-  if (threadIdx.x < kKktUsed) {
-    double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += part[b * kKktSlots + threadIdx.x];
-    tot[threadIdx.x] = s;
-  }
+  const int slot = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nb = slot < kKktRowSlots ? nb_rows : nb_cols;
+  double s = 0.0;
+#pragma unroll 8
+  for (int b = lane; b < nb; b += 32) s += part[b * kKktSlots + slot];
+  s = warp_sum(s);
+  if (lane == 0) tot[slot] = s;
   __syncthreads();
   if (threadIdx.x == 0) {
     const double rel_p = sqrt(tot[0]) / (1.0 + sqrt(tot[2]));
@@ -140,8 +213,8 @@ __global__ void k_kkt_zero(int n, double *v, double *flag) {
 
 }  // namespace
 
-int kkt_blocks(int m, int n) {
-  const int need = ((m > n ? m : n) + kKktThreads - 1) / kKktThreads;
+int kkt_blocks(int rows) {
+  const int need = (rows + kKktThreads - 1) / kKktThreads;
   return need < 1 ? 1 : (need > kKktMaxBlocks ? kKktMaxBlocks : need);
 }
 
@@ -152,18 +225,25 @@ cudaError_t kkt_eval_with_scratch(const rhpdhg_problem *lp, const double *x, con
                                   cudaStream_t st, double *kty, double *part, double *dout,
                                   double *out, bool *bad_index) {
   const int m = lp->m_eq + lp->m_ineq, n = lp->n;
-  const int nb = kkt_blocks(m, n);
+  const int nbc = kkt_blocks(n);
+  // the row kernel's grid is at most the CTAs resident at once: its tiles go round robin, and a
+  // second, partly filled wave would leave SMs idle
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int nbr = std::min(kkt_blocks(m), std::max(1, sms * kKktRowCtas));
   double *flag = dout + kKktFlag;
-  cudaError_t e = launch_kernel(k_kkt_zero, nb, kKktThreads, 0, st, n, kty, flag);
+  e = launch_kernel(k_kkt_zero, nbc, kKktThreads, 0, st, n, kty, flag);
   if (e == cudaSuccess)
-    e = launch_kernel(k_kkt_rows, nb, kKktThreads, 0, st, m, lp->m_eq, n, (long long)lp->nnz,
+    e = launch_kernel(k_kkt_rows, nbr, kKktThreads, 0, st, m, lp->m_eq, n, (long long)lp->nnz,
                (const long long *)lp->row_ptr, lp->col_idx, lp->val, x, y, lp->rhs, kty, part,
                flag);
   if (e == cudaSuccess)
-    e = launch_kernel(k_kkt_cols, nb, kKktThreads, 0, st, n, lp->c, lp->l, lp->u, x, (const double *)kty,
+    e = launch_kernel(k_kkt_cols, nbc, kKktThreads, 0, st, n, lp->c, lp->l, lp->u, x, (const double *)kty,
                part);
   if (e == cudaSuccess)
-    e = launch_kernel(k_kkt_final, 1, 32, 0, st, nb, (const double *)part, lp->obj_offset, dout);
+    e = launch_kernel(k_kkt_final, 1, 32 * kKktUsed, 0, st, nbr, nbc, (const double *)part, lp->obj_offset, dout);
   if (e != cudaSuccess) return e;
   count_launches(4);
   double h[6] = {0};
@@ -218,13 +298,17 @@ extern "C" int rhpdhg_kkt_eval(const rhpdhg_problem *lp, const double *x, const 
   cudaStream_t st = (cudaStream_t)stream;
   double *kty = nullptr, *part = nullptr, *dout = nullptr;
   bool bad_index = false;
-  cudaError_t e = cudaMalloc(&kty, (size_t)n * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&part, (size_t)kKktMaxBlocks * kKktSlotCount * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&dout, 8 * sizeof(double));
+  // scratch from the buffer cache (a cudaMalloc and cudaFree of n doubles per call synchronised the
+  // device and took longer than the evaluation of a mid-size LP)
+  cudaError_t e = buf_alloc((void **)&kty, (size_t)n * sizeof(double));
+  if (e == cudaSuccess)
+    e = buf_alloc((void **)&part, (size_t)kKktMaxBlocks * kKktSlotCount * sizeof(double));
+  if (e == cudaSuccess) e = buf_alloc((void **)&dout, 8 * sizeof(double));
   if (e == cudaSuccess) e = kkt_eval_with_scratch(lp, x, y, st, kty, part, dout, out, &bad_index);
-  cudaFree(kty);
-  cudaFree(part);
-  cudaFree(dout);
+  if (e != cudaSuccess) cudaStreamSynchronize(st);   // nothing in flight uses the scratch
+  buf_release(kty);
+  buf_release(part);
+  buf_release(dout);
   return kkt_finish("rhpdhg_kkt_eval", e, bad_index);
 }
 
