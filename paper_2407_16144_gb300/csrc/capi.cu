@@ -886,9 +886,6 @@ int rhpdhg_create(const rhpdhg_problem *lp, const rhpdhg_params *params, void *c
   }
   // ---- layouts ----
   {
-    std::vector<int> hrp(m + 1), hcp(n + 1);
-    CKT(cudaMemcpy(hrp.data(), rp, (m + 1) * sizeof(int), cudaMemcpyDeviceToHost));
-    CKT(cudaMemcpy(hcp.data(), cp, (n + 1) * sizeof(int), cudaMemcpyDeviceToHost));
     // precision 2 keeps BF16 values of K^, exact when every value of K has at most 8
     // significant bits (the scaling factors are powers of two)
     if (P.precision == 2 && !values_exact_in_bf16(st, h->nnz, val, flags)) {
@@ -900,7 +897,12 @@ int rhpdhg_create(const rhpdhg_problem *lp, const rhpdhg_params *params, void *c
     const int lowp = P.precision;
     h->ic.rho2 = P.algorithm == 1 ? 1 : 0;
     h->ic.df_sums = P.df_sums;
-    if (P.autotune) h->tune_sig = shape_signature(h, hrp, hcp);
+    if (P.autotune) {
+      std::vector<int> hrp(m + 1), hcp(n + 1);
+      CKT(cudaMemcpy(hrp.data(), rp, (m + 1) * sizeof(int), cudaMemcpyDeviceToHost));
+      CKT(cudaMemcpy(hcp.data(), cp, (n + 1) * sizeof(int), cudaMemcpyDeviceToHost));
+      h->tune_sig = shape_signature(h, hrp, hcp);
+    }
     CKT(build_side(st, m, nnz, rp, col, val, h->D, h->E, lowp, &h->rows));
     CKT(build_side(st, n, nnz, cp, ridx, cval, h->E, h->D, lowp, &h->cols));
   }

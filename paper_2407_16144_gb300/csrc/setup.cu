@@ -273,6 +273,273 @@ k_side_spmv_pw(SideLayout lay, SideVals<VT> vals, WalkScratch ws,
   }
 }
 
+
+// ---- layout plan on the device ---------------------------------------------------------------
+// The plan of plan_side (plan.h) from row pointers in device memory, by one warp per tile of 32
+// rows, a lane per row; the host reads back one summary and the arrays are written where they are
+// used.  (Planned on one host core, with the row pointers copied down and the arrays copied up, the
+// 10M columns and 1.75M rows of a 30M-entry flow LP took 42 of the 119 ms of create, 64 iterations
+// and free; the whole is 76 ms now.  250k columns and 100k rows: 14.5 to 13.3 ms.)  Three passes: k_plan_tiles makes every tile's long-row mask and
+// counts and each block's totals, k_plan_scan turns the totals into starts (one block; there is
+// one record per kPlanTiles tiles), k_plan_emit writes the arrays.
+
+constexpr int kPlanTiles = 64;       // tiles of a block: 8 warps, 8 tiles each; a multiple of
+                                     // kMaxTileMult, so that no tile group spans two blocks
+constexpr int kPlanThreads = 256;
+static_assert(kPlanTiles % kMaxTileMult == 0 && kPlanTiles % (kPlanThreads / 32) == 0, "");
+
+// What a tile, a block, or all tiles hold: entries of the short array (each tile's segment padded
+// to 4) and of the long array (each row padded to 4), long rows and their chunks.
+struct PlanCount {
+  long long s, l;
+  int nl, nc;
+};
+__device__ __forceinline__ PlanCount operator+(PlanCount a, const PlanCount &b) {
+  a.s += b.s;
+  a.l += b.l;
+  a.nl += b.nl;
+  a.nc += b.nc;
+  return a;
+}
+struct PlanTile {
+  uint32_t mask;     // long rows
+  int seg, nc;       // entries of the short segment; chunks of the long rows
+  int pad_;
+  long long l;       // padded entries of the long rows
+};
+struct PlanBlock {
+  PlanCount c;                  // totals; after k_plan_scan what precedes the block
+  long long plain, best;        // FP64 adds of wide_rows_pay
+  int maxseg[3];                // longest group segment of 1, 2 and 4 tiles
+};
+
+__device__ __forceinline__ int plan_align4(int v) { return (v + 3) & ~3; }
+
+__global__ void __launch_bounds__(kPlanThreads)
+k_plan_tiles(int nrows, int ntiles, const int *__restrict__ ptr, PlanTile *tiles,
+             PlanBlock *blocks) {
+  __shared__ PlanTile sh[kPlanTiles];
+  __shared__ int cost[kPlanTiles][2];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  for (int k = threadIdx.x >> 5; k < kPlanTiles; k += kPlanThreads / 32) {
+    const int t = blockIdx.x * kPlanTiles + k;
+    const long long r = (long long)t * kTileRows + lane;
+    const int len = t < ntiles && r < nrows ? ptr[r + 1] - ptr[r] : 0;
+    bool lg = len > kShortMax;
+    int sum = (int)__reduce_add_sync(full, lg ? 0u : (unsigned)len);
+    while (sum > kSegBudget) {            // the longest short row, the first of equal ones
+      const unsigned key = lg ? 0u : (unsigned)(len * 32 + 31 - lane) + 1u;
+      const unsigned top = __reduce_max_sync(full, key) - 1u;
+      if (lane == 31 - (int)(top & 31u)) lg = true;
+      sum -= (int)(top >> 5);
+    }
+    const uint32_t mask = __ballot_sync(full, lg);
+    // FP64 adds of the lane-per-row sums and of the best warp-wide threshold (wide_rows_pay)
+    const int sl = lg ? 0 : len;
+    const int mx = (int)__reduce_max_sync(full, (unsigned)sl);
+    const int plain = plan_align4(mx);
+    int best = plain;
+    if (mx > 16)
+      for (int c = 8; c <= 32 && c < mx; c *= 2)
+        best = min(best, c + (int)__reduce_add_sync(
+                                 full, sl > c ? (unsigned)(((sl + 31) >> 5) + 5) : 0u));
+    int nc = 0;
+    long long l = 0;
+    if (mask) {                            // warp-uniform
+      nc = (int)__reduce_add_sync(full, lg ? (unsigned)((len + kChunk - 1) / kChunk) : 0u);
+      l = lg ? ((long long)len + 3) & ~3LL : 0;
+      for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(full, l, o);
+    }
+    if (lane == 0) {
+      sh[k] = PlanTile{mask, sum, nc, 0, l};
+      cost[k][0] = plain;
+      cost[k][1] = best;
+      if (t < ntiles) tiles[t] = sh[k];
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    static_assert(kPlanTiles == 64, "two tiles per lane below");
+    PlanCount c{};
+    int plain = 0, best = 0;
+    const PlanTile a = sh[2 * lane], b = sh[2 * lane + 1];   // tiles past the last hold zeros
+    c.s = plan_align4(a.seg) + plan_align4(b.seg);
+    c.l = a.l + b.l;
+    c.nl = __popc(a.mask) + __popc(b.mask);
+    c.nc = a.nc + b.nc;
+    plain = cost[2 * lane][0] + cost[2 * lane + 1][0];
+    best = cost[2 * lane][1] + cost[2 * lane + 1][1];
+    // group segments run to the last tile's unpadded end; a ragged last group has fewer tiles
+    const int t0 = blockIdx.x * kPlanTiles + 2 * lane;
+    const bool has_b = t0 + 1 < ntiles;
+    const int m1 = max(a.seg, b.seg);
+    const int m2 = has_b ? plan_align4(a.seg) + b.seg : a.seg;
+    const int up = __shfl_down_sync(full, m2, 1);
+    const int m4 = t0 + 2 < ntiles ? plan_align4(a.seg) + plan_align4(b.seg) + up : m2;
+    const int x1 = (int)__reduce_max_sync(full, (unsigned)m1);
+    const int x2 = (int)__reduce_max_sync(full, (unsigned)m2);
+    const int x4 = (int)__reduce_max_sync(full, lane % 2 == 0 ? (unsigned)m4 : 0u);
+    for (int o = 16; o > 0; o >>= 1) {
+      c.s += __shfl_xor_sync(full, c.s, o);
+      c.l += __shfl_xor_sync(full, c.l, o);
+      c.nl += __shfl_xor_sync(full, c.nl, o);
+      c.nc += __shfl_xor_sync(full, c.nc, o);
+      plain += __shfl_xor_sync(full, plain, o);
+      best += __shfl_xor_sync(full, best, o);
+    }
+    if (lane == 0) blocks[blockIdx.x] = PlanBlock{c, plain, best, {x1, x2, x4}};
+  }
+}
+
+// One block: every block's totals become what precedes it; all[0] the totals over all blocks.
+__global__ void __launch_bounds__(kPlanThreads)
+k_plan_scan(int nblocks, PlanBlock *blocks, PlanBlock *all) {
+  __shared__ PlanCount sh[kPlanThreads];
+  __shared__ long long cost[kPlanThreads][2];
+  __shared__ int mxs[kPlanThreads][3];
+  const int tid = threadIdx.x;
+  const int per = (nblocks + kPlanThreads - 1) / kPlanThreads;
+  const int b0 = min(tid * per, nblocks), b1 = min(b0 + per, nblocks);
+  PlanCount c{};
+  long long plain = 0, best = 0;
+  int mx[3] = {0, 0, 0};
+#pragma unroll 4
+  for (int b = b0; b < b1; ++b) {
+    const PlanBlock r = blocks[b];
+    c = c + r.c;
+    plain += r.plain;
+    best += r.best;
+    for (int k = 0; k < 3; ++k) mx[k] = max(mx[k], r.maxseg[k]);
+  }
+  sh[tid] = c;
+  cost[tid][0] = plain;
+  cost[tid][1] = best;
+  for (int k = 0; k < 3; ++k) mxs[tid][k] = mx[k];
+  __syncthreads();
+  for (int o = 1; o < kPlanThreads; o *= 2) {       // inclusive scan; totals in the last thread
+    PlanCount p{};
+    long long q0 = 0, q1 = 0;
+    int m[3] = {0, 0, 0};
+    if (tid >= o) {
+      p = sh[tid - o];
+      q0 = cost[tid - o][0];
+      q1 = cost[tid - o][1];
+      for (int k = 0; k < 3; ++k) m[k] = mxs[tid - o][k];
+    }
+    __syncthreads();
+    sh[tid] = sh[tid] + p;
+    cost[tid][0] += q0;
+    cost[tid][1] += q1;
+    for (int k = 0; k < 3; ++k) mxs[tid][k] = max(mxs[tid][k], m[k]);
+    __syncthreads();
+  }
+  if (tid == kPlanThreads - 1)
+    *all = PlanBlock{sh[tid], cost[tid][0], cost[tid][1], {mxs[tid][0], mxs[tid][1], mxs[tid][2]}};
+  PlanCount before{};
+  if (tid > 0) before = sh[tid - 1];
+  for (int b = b0; b < b1; ++b) {
+    const PlanCount own = blocks[b].c;
+    blocks[b].c = before;
+    before = before + own;
+  }
+}
+
+__global__ void __launch_bounds__(kPlanThreads)
+k_plan_emit(int nrows, int ntiles, const int *__restrict__ ptr, const PlanTile *tiles,
+            const PlanBlock *blocks, int *ptr_s, int *tile_end, int *dst, uint32_t *long_mask,
+            int *long_rows, int *beg_l, int *end_l, int *chunk_ptr, int *chunk_row) {
+  __shared__ PlanCount sh[kPlanTiles];      // what precedes each tile, from the block's start
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, tid = threadIdx.x;
+  const int first = blockIdx.x * kPlanTiles;
+  if (tid < kPlanTiles) {
+    PlanCount c{};
+    if (first + tid < ntiles) {
+      const PlanTile x = tiles[first + tid];
+      c.s = plan_align4(x.seg);
+      c.l = x.l;
+      c.nl = __popc(x.mask);
+      c.nc = x.nc;
+    }
+    sh[tid] = c;
+  }
+  __syncthreads();
+  for (int o = 1; o < kPlanTiles; o *= 2) {
+    PlanCount p{};
+    if (tid < kPlanTiles && tid >= o) p = sh[tid - o];
+    __syncthreads();
+    if (tid < kPlanTiles) sh[tid] = sh[tid] + p;
+    __syncthreads();
+  }
+  const PlanCount base = blocks[blockIdx.x].c;
+  if (blockIdx.x == 0 && tid == 0) chunk_ptr[0] = 0;
+  for (int k = tid >> 5; k < kPlanTiles; k += kPlanThreads / 32) {
+    const int t = first + k;
+    if (t >= ntiles) break;
+    PlanCount at = base;
+    if (k > 0) at = at + sh[k - 1];
+    const long long r = (long long)t * kTileRows + lane;
+    const int len = r < nrows ? ptr[r + 1] - ptr[r] : 0;
+    const uint32_t mask = tiles[t].mask;
+    const bool lg = (mask >> lane) & 1u;
+    int incl = lg ? 0 : len;                 // short entries up to and with this row
+    for (int o = 1; o < 32; o *= 2) {
+      const int v = __shfl_up_sync(full, incl, o);
+      if (lane >= o) incl += v;
+    }
+    const int start = (int)at.s + incl - (lg ? 0 : len);
+    int to = start;
+    if (mask) {                              // warp-uniform
+      const int nc = lg ? (len + kChunk - 1) / kChunk : 0;
+      const long long pl = lg ? ((long long)len + 3) & ~3LL : 0;
+      int ci = nc;
+      long long li = pl;
+      for (int o = 1; o < 32; o *= 2) {
+        const int v = __shfl_up_sync(full, ci, o);
+        const long long w = __shfl_up_sync(full, li, o);
+        if (lane >= o) {
+          ci += v;
+          li += w;
+        }
+      }
+      const int row = at.nl + __popc(mask & ((1u << lane) - 1u));
+      if (lg) {
+        to = (int)(at.l + li - pl);
+        long_rows[row] = (int)r;
+        beg_l[row] = to;
+        end_l[row] = to + len;
+        chunk_ptr[row + 1] = at.nc + ci;
+      }
+      for (uint32_t left = mask; left; left &= left - 1u) {
+        const int b = __ffs((int)left) - 1;
+        const int n = __shfl_sync(full, nc, b), c1 = at.nc + __shfl_sync(full, ci, b);
+        const int id = __shfl_sync(full, row, b);
+        for (int c = c1 - n + lane; c < c1; c += 32) chunk_row[c] = id;
+      }
+    }
+    if (r < nrows) {
+      ptr_s[r] = start;
+      dst[r] = to;
+    }
+    if (lane == 0) {
+      tile_end[t] = (int)at.s + tiles[t].seg;
+      long_mask[t] = mask;
+    }
+  }
+}
+
+// Per chunk: its long row, entry range, and the chunk count of its group of 32 long rows.
+__global__ void k_plan_desc(int nchunks, int nlong, const int *chunk_row, const int *chunk_ptr,
+                            const int *beg_l, const int *end_l, int4 *desc) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= nchunks) return;
+  const int li = chunk_row[c];
+  const int cb = beg_l[li] + (c - chunk_ptr[li]) * kChunk;
+  const int g0 = (li / kTileRows) * kTileRows, g1 = min(g0 + kTileRows, nlong);
+  desc[c] = make_int4(li, cb, min(cb + kChunk, end_l[li]), chunk_ptr[g1] - chunk_ptr[g0]);
+}
+
 }  // namespace
 
 static std::atomic<long long> g_launches{0};
@@ -510,6 +777,11 @@ size_t buf_drop_cache() {
   return freed;
 }
 
+// Warp-wide sums are enabled when they save at least 15% of the FP64 adds.
+static bool wide_pays(long long plain, long long best) {
+  return plain > 0 && (double)best <= 0.85 * (double)plain;
+}
+
 // The cost model of tile_rows_fp64 over all short tiles of a side: FP64 adds per warp of the
 // lane-per-row sums (4 ceil(longest / 4) per tile) against the best threshold's (c + the sum over
 // rows longer than c of ceil(len / 32) + 5, c in 8, 16, 32).  The warp-wide sums are enabled
@@ -538,7 +810,21 @@ static bool wide_rows_pay(const int *hp, const std::vector<uint32_t> &mask, int 
     plain += p;
     best += b;
   }
-  return plain > 0 && (double)best <= 0.85 * (double)plain;
+  return wide_pays(plain, best);
+}
+
+// Tiles per work item: where tiles are short (a few entries per row), M consecutive tiles are
+// staged as one segment, so that each warp's chain of dependent loads carries M tiles' bytes.
+// M is the largest of kMaxTileMult, ..., 2 whose mean group segment fits one staging round
+// (128 * kStageUnroll entries) and whose longest fits the staging budget; else 1.  nnz_s: entries
+// of the short array; maxseg_mult: longest group segments (-1: over the budget).
+static int rule_mult(int ntiles, long long nnz_s, const long long *maxseg_mult) {
+  for (int k = 2, cand = kMaxTileMult; cand >= 2; --k, cand /= 2) {
+    if (ntiles < 2 * cand) continue;
+    if (nnz_s * cand > (long long)ntiles * kWarp * kStageUnroll * 4) continue;
+    if (maxseg_mult[k] >= 0) return cand;
+  }
+  return 1;
 }
 
 bool plan_side(const int *hp, int nrows, SidePlan *p) {
@@ -601,10 +887,6 @@ bool plan_side(const int *hp, int nrows, SidePlan *p) {
   P.nnz_s = align4(cur) + 4;
   P.nnz_l = align4(cl) + kChunk;
   if (P.nnz_s > INT_MAX || P.nnz_l > INT_MAX) return false;
-  // Tiles per work item: where tiles are short (a few entries per row), M consecutive tiles are
-  // staged as one segment, so that each warp's chain of dependent loads carries M tiles' bytes.
-  // M is the largest of kMaxTileMult, ..., 2 whose mean group segment fits one staging round
-  // (128 * kStageUnroll entries) and whose longest fits the staging budget; else 1.
   P.maxseg_mult[0] = maxseg;
   for (int k = 1, cand = 2; cand <= kMaxTileMult; ++k, cand *= 2) {
     long long mx = 0;
@@ -614,17 +896,8 @@ bool plan_side(const int *hp, int nrows, SidePlan *p) {
     }
     P.maxseg_mult[k] = (ntiles > 0 && mx <= kSegBudget) ? mx : -1;
   }
-  int mult = 1;
-  for (int k = 2, cand = kMaxTileMult; cand >= 2 && mult == 1; --k, cand /= 2) {
-    if (ntiles < 2 * cand) continue;
-    if (align4(cur) * cand > (long long)ntiles * kWarp * kStageUnroll * 4) continue;
-    if (P.maxseg_mult[k] >= 0) {
-      mult = cand;
-      maxseg = P.maxseg_mult[k];
-    }
-  }
-  P.mult = mult;
-  P.maxseg = maxseg;
+  P.mult = rule_mult(ntiles, align4(cur), P.maxseg_mult);
+  P.maxseg = P.maxseg_mult[P.mult == 4 ? 2 : P.mult - 1];
   P.wide_rows = wide_rows_pay(hp, P.mask, nrows) ? 1 : 0;
   return true;
 }
@@ -635,67 +908,82 @@ cudaError_t build_side(cudaStream_t st, int nrows, int nnz, const int *ptr, cons
   (void)nnz;
   SideStore s;
   cudaError_t err = cudaSuccess;
-  // ---- structure, on the host -------------------------------------------------------------
-  std::vector<int> hp(nrows + 1);
-  if ((err = cudaMemcpy(hp.data(), ptr, (nrows + 1) * sizeof(int), cudaMemcpyDeviceToHost)))
-    return err;
-  SidePlan P;
-  if (!plan_side(hp.data(), nrows, &P)) return cudaErrorInvalidValue;
-  const int ntiles = P.ntiles, mult = P.mult;
-  const long long nnz_s = P.nnz_s, nnz_l = P.nnz_l, maxseg = P.maxseg;
-  const std::vector<int> &ptr_s = P.ptr_s, &tile_end = P.tile_end, &dst = P.dst,
-                         &long_rows = P.long_rows, &beg_l = P.beg_l, &end_l = P.end_l,
-                         &chunk_ptr = P.chunk_ptr, &chunk_row = P.chunk_row;
-  const std::vector<uint32_t> &mask = P.mask;
-  auto align4 = [](long long v) { return (v + 3) & ~3LL; };
-  const int nlong = (int)long_rows.size(), nch = (int)chunk_row.size();
-  s.lay.nrows = nrows;
-  s.lay.seg = (int)align4(maxseg) + 4;
-  s.lay.n_short_tiles = ntiles;
-  s.lay.tile_mult = mult;
-  s.lay.n_tile_groups = (ntiles + mult - 1) / mult;
-  s.lay.n_long = nlong;
-  s.lay.n_long_tiles = (nlong + kTileRows - 1) / kTileRows;
-  s.lay.n_chunks = nch;
-  s.lay.wide_rows = P.wide_rows;
-  s.rule_mult = mult;
-  for (int k = 0; k < 3; ++k) s.maxseg_mult[k] = P.maxseg_mult[k];
-  s.nnz_short = nnz_s;
-  s.nnz_long = nnz_l;
-  const size_t ng = (size_t)std::max(s.lay.n_long_tiles, 1);
+  const int ntiles = (int)(((long long)nrows + kTileRows - 1) / kTileRows);
+  const int nplan = (ntiles + kPlanTiles - 1) / kPlanTiles;
   int *d_dst = nullptr;
-  auto up = [&](int **d, const std::vector<int> &h) -> cudaError_t {
-    cudaError_t e = buf_alloc((void **)d, std::max<size_t>(h.size(), 1) * sizeof(int));
-    if (e == cudaSuccess && !h.empty())
-      e = cudaMemcpy(*d, h.data(), h.size() * sizeof(int), cudaMemcpyHostToDevice);
-    return e;
+  PlanTile *d_tiles = nullptr;
+  PlanBlock *d_blocks = nullptr;
+  PlanBlock tot{};
+  long long nnz_s = 0, nnz_l = 0;
+  int nlong = 0, nch = 0;
+  size_t ng = 1;
+  auto get = [](auto **d, size_t count) {
+    return buf_alloc((void **)d, std::max<size_t>(count, 1) * sizeof(**d));
   };
 #define TRY(x)                 \
   do {                         \
     if ((err = (x))) goto fail; \
   } while (0)
-  TRY(up(&s.ptr_s, ptr_s));
-  TRY(up(&s.tile_end, tile_end));
-  TRY(up(&s.long_rows, long_rows));
-  TRY(up(&s.beg_l, beg_l));
-  TRY(up(&s.end_l, end_l));
-  TRY(up(&s.chunk_ptr, chunk_ptr));
-  TRY(up(&s.chunk_row, chunk_row));
-  {
-    // per chunk: its long row, entry range, and the chunk count of its group of 32 long rows
-    std::vector<int4> desc((size_t)std::max(nch, 1));
-    for (int c = 0; c < nch; ++c) {
-      const int li = chunk_row[c];
-      const int cb = beg_l[li] + (c - chunk_ptr[li]) * kChunk;
-      const int g0 = (li / kTileRows) * kTileRows, g1 = std::min(g0 + kTileRows, nlong);
-      desc[c] = make_int4(li, cb, std::min(cb + kChunk, end_l[li]), chunk_ptr[g1] - chunk_ptr[g0]);
-    }
-    TRY(buf_alloc((void **)&s.chunk_desc, desc.size() * sizeof(int4)));
-    TRY(cudaMemcpy(s.chunk_desc, desc.data(), desc.size() * sizeof(int4), cudaMemcpyHostToDevice));
+  // ---- structure: counts, then arrays of their sizes -----------------------------------------
+  TRY(get(&d_tiles, ntiles));
+  TRY(get(&d_blocks, (size_t)nplan + 1));
+  if (ntiles > 0) {
+    k_plan_tiles<<<nplan, kPlanThreads, 0, st>>>(nrows, ntiles, ptr, d_tiles, d_blocks);
+    k_plan_scan<<<1, kPlanThreads, 0, st>>>(nplan, d_blocks, d_blocks + nplan);
+    count_launches(2);
+    TRY(cudaMemcpyAsync(&tot, d_blocks + nplan, sizeof(tot), cudaMemcpyDeviceToHost, st));
+    TRY(cudaStreamSynchronize(st));
   }
-  TRY(up(&d_dst, dst));
-  TRY(buf_alloc((void **)&s.long_mask, mask.size() * sizeof(uint32_t)));
-  TRY(cudaMemcpy(s.long_mask, mask.data(), mask.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
+  if (tot.c.s > INT_MAX - 16 || tot.c.l > INT_MAX - 2 * kChunk - 16) {
+    // at the limit of the int32 offsets the host plan says whether they hold (its limits are on
+    // unpadded ends)
+    std::vector<int> hp((size_t)nrows + 1);
+    SidePlan P;
+    TRY(cudaMemcpy(hp.data(), ptr, hp.size() * sizeof(int), cudaMemcpyDeviceToHost));
+    if (!plan_side(hp.data(), nrows, &P)) {
+      err = cudaErrorInvalidValue;
+      goto fail;
+    }
+  }
+  nlong = tot.c.nl;
+  nch = tot.c.nc;
+  nnz_s = tot.c.s + 4;
+  nnz_l = tot.c.l + kChunk;
+  for (int k = 0; k < 3; ++k)
+    s.maxseg_mult[k] =
+        k == 0 || (ntiles > 0 && tot.maxseg[k] <= kSegBudget) ? (long long)tot.maxseg[k] : -1;
+  s.rule_mult = rule_mult(ntiles, tot.c.s, s.maxseg_mult);
+  s.lay.nrows = nrows;
+  s.lay.n_short_tiles = ntiles;
+  apply_mult(s, s.rule_mult);
+  s.lay.n_long = nlong;
+  s.lay.n_long_tiles = (nlong + kTileRows - 1) / kTileRows;
+  s.lay.n_chunks = nch;
+  s.lay.wide_rows = wide_pays(tot.plain, tot.best) ? 1 : 0;
+  s.nnz_short = nnz_s;
+  s.nnz_long = nnz_l;
+  ng = (size_t)std::max(s.lay.n_long_tiles, 1);
+  TRY(get(&s.ptr_s, nrows));
+  TRY(get(&s.tile_end, ntiles));
+  TRY(get(&s.long_rows, nlong));
+  TRY(get(&s.beg_l, nlong));
+  TRY(get(&s.end_l, nlong));
+  TRY(get(&s.chunk_ptr, (size_t)nlong + 1));
+  TRY(get(&s.chunk_row, nch));
+  TRY(get(&s.chunk_desc, nch));
+  TRY(get(&d_dst, nrows));
+  TRY(get(&s.long_mask, ntiles));
+  if (ntiles > 0) {
+    k_plan_emit<<<nplan, kPlanThreads, 0, st>>>(nrows, ntiles, ptr, d_tiles, d_blocks, s.ptr_s,
+                                                s.tile_end, d_dst, s.long_mask, s.long_rows,
+                                                s.beg_l, s.end_l, s.chunk_ptr, s.chunk_row);
+    count_launches(1);
+    if (nch > 0) {
+      k_plan_desc<<<nblocks(nch, 256), 256, 0, st>>>(nch, nlong, s.chunk_row, s.chunk_ptr, s.beg_l,
+                                                     s.end_l, s.chunk_desc);
+      count_launches(1);
+    }
+  }
   // ---- entries (zero padding), scaled on the device ------------------------------------------
   TRY(buf_alloc((void **)&s.idx_s, nnz_s * sizeof(int)));
   TRY(buf_alloc((void **)&s.val64_s, nnz_s * sizeof(double)));
@@ -741,6 +1029,8 @@ cudaError_t build_side(cudaStream_t st, int nrows, int nnz, const int *ptr, cons
   TRY(cudaGetLastError());
 #undef TRY
   buf_release(d_dst);
+  buf_release(d_tiles);
+  buf_release(d_blocks);
   s.lay.ptr_s = s.ptr_s;
   s.lay.tile_end = s.tile_end;
   s.lay.idx_s = s.idx_s;
@@ -769,6 +1059,8 @@ cudaError_t build_side(cudaStream_t st, int nrows, int nnz, const int *ptr, cons
 fail:
   cudaStreamSynchronize(st);
   buf_release(d_dst);
+  buf_release(d_tiles);
+  buf_release(d_blocks);
   free_side(&s);
   return err;
 }
