@@ -945,7 +945,8 @@ int rhpdhg_create(const rhpdhg_problem *lp, const rhpdhg_params *params, void *c
   // v <- K^T K^ v / ||K^T K^ v|| from v = 1/sqrt(n); each step is two fused products (the
   // normalisation rides on the next product's input scale), then sigma = ||K^ v||.
   {
-    double *v = nullptr, *w = nullptr, *um = nullptr, *pp = nullptr, *ss = nullptr;
+    void *v = nullptr, *w = nullptr, *um = nullptr;
+    double *pp = nullptr, *ss = nullptr;
     unsigned int *tk = nullptr;
     // FP64 handles in FP64; mixed-precision handles in their own value precision with FP32
     // products and row sums (the step keeps its 10% margin: eta sigma_max = 0.9 (1 + O(1e-6)))
@@ -953,14 +954,16 @@ int rhpdhg_create(const rhpdhg_problem *lp, const rhpdhg_params *params, void *c
     const int gr = side_spmv_pw_grid(h->rows, lowp, h->sm_count);
     const int gc = side_spmv_pw_grid(h->cols, lowp, h->sm_count);
     const int gmax = std::max(gr, gc);
-    CKT(dalloc(&v, n));
-    CKT(dalloc(&w, n));
-    CKT(dalloc(&um, m));
+    const size_t vb = lowp ? sizeof(float) : sizeof(double);
+    CKT(buf_alloc(&v, (size_t)n * vb));
+    CKT(buf_alloc(&w, (size_t)n * vb));
+    CKT(buf_alloc(&um, (size_t)m * vb));
     CKT(dalloc(&pp, (size_t)gmax * kMaxPartials));
     CKT(dalloc(&ss, 8));
     CKT(dalloc(&tk, 1));
     CKT(cudaMemsetAsync(tk, 0, sizeof(unsigned int), st));
-    fill(st, n, 1.0 / std::sqrt((double)n), v);
+    if (lowp) fill_f32(st, n, (float)(1.0 / std::sqrt((double)n)), (float *)v);
+    else fill(st, n, 1.0 / std::sqrt((double)n), (double *)v);
     const double *scale = nullptr;       // v is already normalised
     for (int it = 0; it < P.power_iters; ++it) {
       side_spmv_pw(st, h->rows, lowp, v, scale, um, pp, tk, ss + 2, gr);

@@ -135,17 +135,18 @@ int tile_grid(const SideLayout &lay, int sm_count, int blocks_per_sm);
 // out = side * src   (plain product, FP64)
 void side_spmv(cudaStream_t st, const SideStore &side, const double *src, double *out, int grid);
 // Power-iteration product: out = side * (src * in_scale[0]) and ss = (||out||^2, 1/||out||);
-// lowp 0: FP64 values, products and sums; 1 / 2: the side's FP32 / BF16 values with FP32 products
-// and row sums (mixed-precision handles); the norm is an FP64 sum in every case.
-// part holds grid * kMaxPartials doubles, ticket a zeroed counter.
-void side_spmv_pw(cudaStream_t st, const SideStore &side, int lowp, const double *src,
-                  const double *in_scale, double *out, double *part, unsigned int *ticket,
+// lowp 0: FP64 vectors, values, products and sums; 1 / 2: FP32 vectors and the side's FP32 / BF16
+// values with FP32 products and row sums (mixed-precision handles); the norm is an FP64 sum in
+// every case.  part holds grid * kMaxPartials doubles, ticket a zeroed counter.
+void side_spmv_pw(cudaStream_t st, const SideStore &side, int lowp, const void *src,
+                  const double *in_scale, void *out, double *part, unsigned int *ticket,
                   double *ss, int grid);
 int side_spmv_pw_grid(const SideStore &side, int lowp, int sm_count);
 // deterministic sum of squares -> *out (device scalar); tmp holds >= 1024 doubles
 void sumsq(cudaStream_t st, int n, const double *x, double *out, double *tmp);
 // v = w / sqrt(*ss)
 void fill(cudaStream_t st, int n, double v, double *x);
+void fill_f32(cudaStream_t st, int n, float v, float *x);
 // y = a .* x (elementwise), optionally y = x ./ a when div = 1
 void vmul(cudaStream_t st, int n, const double *a, const double *x, double *y, int div);
 // x = clamp(x, l, u)

@@ -207,7 +207,8 @@ __global__ void k_sum_final(int nparts, const double *part, double *out) {
   if (threadIdx.x == 0) *out = sh[0];
 }
 
-__global__ void k_fill(int n, double v, double *x) {
+template <typename T>
+__global__ void k_fill(int n, T v, T *x) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) x[i] = v;
 }
@@ -236,14 +237,18 @@ k_side_spmv(SideLayout lay, SideVals<double> vals, WalkScratch ws,
 // One product of the power iteration on K^T K^: out = side * (src * in_scale[0]) (in_scale NULL:
 // 1), plus ss[0] = ||out||^2 and ss[1] = 1 / ||out|| (0 for a zero vector) from the grid's
 // deterministic ticket reduction.  The next product reads ss + 1 as its input scale, so the
-// normalisation v = w / ||w|| costs no launch of its own.  PT is the product and row-sum type:
-// FP64 with the FP64 values; FP32 with the FP32 or BF16 values of a mixed-precision handle, where
-// the input scale is applied to each row's sum (in FP64) instead of to every gathered entry and
-// the norm is still an FP64 sum.
+// normalisation v = w / ||w|| costs no launch of its own.  PT is the vector, product and row-sum
+// type: FP64 with the FP64 values; FP32 with the FP32 or BF16 values of a mixed-precision handle,
+// where the input scale is applied to each row's sum (in FP64) instead of to every gathered entry
+// and the norm is still an FP64 sum, of the rows before they are rounded to the FP32 vector.  (An
+// FP64 vector, rounded as it was gathered, gave the same bits with twice the vector traffic:
+// create, 64
+// iterations and free of a 30M-entry LP in BF16 76.3 to 69.1 ms, of a 2.5M-entry LP in FP32 13.3 to
+// 12.8 ms.)
 template <typename VT, typename PT>
 __global__ void __launch_bounds__(kBlockThreads)
 k_side_spmv_pw(SideLayout lay, SideVals<VT> vals, WalkScratch ws,
-               const double *__restrict__ src, const double *in_scale, double *out, double *part,
+               const PT *__restrict__ src, const double *in_scale, PT *out, double *part,
                unsigned int *ticket, double *ss) {
   extern __shared__ double smem[];
   PT *my = reinterpret_cast<PT *>(smem) + (threadIdx.x >> 5) * lay.seg;
@@ -255,11 +260,11 @@ k_side_spmv_pw(SideLayout lay, SideVals<VT> vals, WalkScratch ws,
   al.zero();
   auto epi = [&](int row, PT dot, bool lg) {
     const double o = (double)dot * post;
-    out[row] = o;
+    out[row] = (PT)o;
     if (lg) al.s[0] += o * o;
     else a.s[0] += o * o;
   };
-  auto gather = [&](int j) { return kF64 ? PT(src[j] * sc) : PT(src[j]); };
+  auto gather = [&](int j) { return kF64 ? PT(src[j] * sc) : src[j]; };
   auto gdone = [&](int grp) { store_group(al, 0x1u, ws.group_part, grp); };
   walk_tiles<VT, PT>(lay, vals, gather, my, ws, epi, gdone);
   if (cta_reduce_and_ticket(a, 0x1u, 0u, 0u, part, ticket)) {
@@ -272,7 +277,6 @@ k_side_spmv_pw(SideLayout lay, SideVals<VT> vals, WalkScratch ws,
     }
   }
 }
-
 
 // ---- layout plan on the device ---------------------------------------------------------------
 // The plan of plan_side (plan.h) from row pointers in device memory, by one warp per tile of 32
@@ -1117,19 +1121,22 @@ static int pw_smem(const SideStore &side, int lowp) {
   return kBlockWarps * side.lay.seg * (lowp ? (int)sizeof(float) : (int)sizeof(double));
 }
 
-void side_spmv_pw(cudaStream_t st, const SideStore &side, int lowp, const double *src,
-                  const double *in_scale, double *out, double *part, unsigned int *ticket,
+void side_spmv_pw(cudaStream_t st, const SideStore &side, int lowp, const void *src,
+                  const double *in_scale, void *out, double *part, unsigned int *ticket,
                   double *ss, int grid) {
   const int smem = pw_smem(side, lowp);
+  const float *sf = (const float *)src;
+  float *of = (float *)out;
   if (lowp == 2)
     k_side_spmv_pw<__nv_bfloat16, float><<<grid, kBlockThreads, smem, st>>>(
-        side.lay, side.v16, side.wa, src, in_scale, out, part, ticket, ss);
+        side.lay, side.v16, side.wa, sf, in_scale, of, part, ticket, ss);
   else if (lowp == 1)
     k_side_spmv_pw<float, float><<<grid, kBlockThreads, smem, st>>>(
-        side.lay, side.v32, side.wa, src, in_scale, out, part, ticket, ss);
+        side.lay, side.v32, side.wa, sf, in_scale, of, part, ticket, ss);
   else
     k_side_spmv_pw<double, double><<<grid, kBlockThreads, smem, st>>>(
-        side.lay, side.v64, side.wa, src, in_scale, out, part, ticket, ss);
+        side.lay, side.v64, side.wa, (const double *)src, in_scale, (double *)out, part, ticket,
+        ss);
   count_launches(1);
 }
 
@@ -1162,6 +1169,11 @@ void sumsq(cudaStream_t st, int n, const double *x, double *out, double *tmp) {
 }
 
 void fill(cudaStream_t st, int n, double v, double *x) {
+  k_fill<<<nblocks(n, 256), 256, 0, st>>>(n, v, x);
+  count_launches(1);
+}
+
+void fill_f32(cudaStream_t st, int n, float v, float *x) {
   k_fill<<<nblocks(n, 256), 256, 0, st>>>(n, v, x);
   count_launches(1);
 }
