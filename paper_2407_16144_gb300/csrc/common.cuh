@@ -87,7 +87,7 @@ struct SideLayout {
   int tile_mult = 1;         // consecutive short tiles per work item (1 .. kMaxTileMult)
   int walk = 0;              // instantiation of the ordinary mixed kernels' walk (kWalk*)
   int cta_warps = kBlockWarps;  // warps per CTA of this side's iteration kernels (host only)
-  int wide_rows = 0;         // FP64 walks sum a tile's longest rows warp-wide (tile_rows_fp64)
+  int wide_rows = 0;         // reported: skewed tiles (wide_rows_pay in setup.cu)
   int n_tile_groups = 0;     // ceil(n_short_tiles / tile_mult)
   __host__ __device__ int total_items() const { return n_chunks + n_tile_groups; }
 };
@@ -251,6 +251,20 @@ __device__ __forceinline__ bool dbl_pos(double x) {
 __device__ __forceinline__ bool dbl_neg(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull;
+}
+// fmax(x, 0) and fmin(x, 0)
+__device__ __forceinline__ double dbl_pos_part(double x) { return dbl_pos(x) ? x : 0.0; }
+__device__ __forceinline__ double dbl_neg_part(double x) { return dbl_neg(x) ? x : 0.0; }
+// fmin(fmax(x, l), u) for l <= u, neither of them NaN
+__device__ __forceinline__ double dbl_clamp(double x, double l, double u) {
+  auto key = [](double v) {               // increases with v (-0 below +0)
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+  };
+  const long long k = key(x);
+  double r = k < key(l) ? l : x;
+  r = k > key(u) ? u : r;
+  return dbl_nan(x) ? l : r;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -804,7 +818,10 @@ __device__ __forceinline__ void walk_chunk(const SideLayout &lay, const SideVals
 // adds an equal run of L consecutive entries (L odd: no shared-memory bank conflicts), writing its
 // running sum over the last entry of every row, and of the run, that it completes; lane r then adds
 // the one or few partial sums of its row, in entry order.  That is L + (runs a row spans) adds for
-// the warp.  Where no row is longer than that, one lane per row is kept.
+// the warp.  Where no row is longer than that, one lane per row is kept.  Measured with the integer
+// comparisons above, FP64 iterations against lane-per-row sums (or, on skewed sides, sums of the
+// longest rows by the whole warp): 2.5M entries with power-law columns 112 to 93 us, flow LP of 30M
+// entries 797 to 703 us, 150k even entries 36 to 34 us.
 template <typename PT>
 __device__ __forceinline__ PT balanced_row_sum(PT *s, int len, int b, int e) {
   const unsigned full = 0xffffffffu;
@@ -857,40 +874,24 @@ __device__ __forceinline__ PT balanced_row_sum(PT *s, int len, int b, int e) {
   return t;
 }
 
-// FP64 tiles: the FP64 pipe is narrow, and lane-per-row sums issue as many FP64 adds per warp as
-// the tile's longest row has entries, with the other lanes masked.  Rows longer than a threshold
-// T are therefore summed by the whole warp (lane-strided partial sums and a shuffle tree, about
-// len/32 + 5 adds per row), the rest lane per row as in tile_rows.  T is the candidate among 8,
-// 16, 32 and the longest row that minimises the warp's FP64 adds, 4 ceil(T / 4) + the sum over
-// rows longer than T of (ceil(len / 32) + 5) (one warp reduction per candidate); a tile whose rows
-// have at most 16 entries keeps T = its longest row.  Rows at or below T are summed exactly as
-// tile_rows sums them.  Used only on sides where the same cost model, evaluated over all tiles at
-// set-up, saves FP64 adds (SideLayout::wide_rows); elsewhere tile_rows keeps lane-per-row sums.
-template <typename Epi>
-__device__ __forceinline__ void tile_rows_fp64(const double *smem, int row0, int nr, int rb,
-                                               int re, int seg_b, uint32_t lm, Epi &epi) {
-  const unsigned full = 0xffffffffu;
+// Sums the rows of a short tile from the staged products smem[0, ...) (staged from seg_b on) and
+// runs their epilogues, lane r row r (rows marked long in lm are skipped).  FP64 tiles balance the
+// additions over the lanes (balanced_row_sum); FP32 tiles, whose pipe is wide, sum lane per row
+// with four interleaved accumulators, each lane going on to its epilogue as soon as its row is
+// summed, so that its loads overlap the other lanes' sums.
+template <typename PT, typename Epi>
+__device__ __forceinline__ void tile_rows(PT *smem, int row0, int nr, int rb, int re,
+                                          int seg_b, uint32_t lm, Epi &epi) {
   const int lane = threadIdx.x & 31;
   const bool act = lane < nr && !((lm >> lane) & 1u);
-  const int len = act ? re - rb : 0;           // at most kShortMax
-  const int mx = (int)__reduce_max_sync(full, (unsigned)len);
-  int T = mx;
-  if (mx > 16) {
-    int best = (mx + 3) & ~3;
-    const int wadds = ((len + 31) >> 5) + 5;   // this row's adds when summed by the warp
-#pragma unroll
-    for (int c = 8; c <= 32; c *= 2) {
-      if (c >= mx) break;
-      const int cost = c + (int)__reduce_add_sync(full, len > c ? (unsigned)wadds : 0u);
-      if (cost < best) {
-        best = cost;
-        T = c;
-      }
-    }
-  }
-  double dot = 0.0;
-  if (act && len <= T) {
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+  if constexpr (sizeof(PT) == sizeof(double)) {
+    const int tb = __shfl_sync(0xffffffffu, rb, 0), te = __shfl_sync(0xffffffffu, re, nr - 1);
+    // (a long row's short range is empty; lanes past the last row take an empty one at the end)
+    const int b = lane < nr ? rb - tb : te - tb, e = lane < nr ? re - tb : te - tb;
+    const PT dot = balanced_row_sum(smem + (tb - seg_b), te - tb, b, e);
+    if (act) epi(row0 + lane, dot, false);
+  } else if (act) {
+    PT s0 = PT(0), s1 = PT(0), s2 = PT(0), s3 = PT(0);
     int p = rb - seg_b;
     const int pe = re - seg_b;
     for (; p + 4 <= pe; p += 4) {
@@ -902,57 +903,9 @@ __device__ __forceinline__ void tile_rows_fp64(const double *smem, int row0, int
     if (p < pe) s0 += smem[p];
     if (p + 1 < pe) s1 += smem[p + 1];
     if (p + 2 < pe) s2 += smem[p + 2];
-    dot = (s0 + s1) + (s2 + s3);
-  }
-  unsigned big = __ballot_sync(full, act && len > T);
-  while (big) {
-    const int r = __ffs(big) - 1;
-    big &= big - 1;
-    const int b = __shfl_sync(full, rb, r) - seg_b, e = __shfl_sync(full, re, r) - seg_b;
-    double s = 0.0;
-    for (int p = b + lane; p < e; p += 32) s += smem[p];
-    s = warp_sum(s);
-    if (lane == r) dot = s;
-  }
-  // one converged epilogue pass (split into the short rows' and the long rows' lanes, the FP64
-  // epilogue issued twice and measured slower)
-  if (act) epi(row0 + lane, dot, false);
-}
-
-// Lane r of a short tile sums row r's staged products smem[rb - seg_b, re - seg_b) with four
-// interleaved accumulators and runs its epilogue (rows marked long in lm are skipped).  FP64
-// tiles go to tile_rows_fp64.
-template <typename PT, typename Epi>
-__device__ __forceinline__ void tile_rows(const PT *smem, int row0, int nr, int rb, int re,
-                                          int seg_b, uint32_t lm, bool wide, Epi &epi) {
-  // (without the warp-wide sums each lane goes on to its epilogue as soon as its row is summed,
-  // so its loads overlap the other lanes' sums)
-  if constexpr (sizeof(PT) == sizeof(double)) {
-    if (wide) {
-      tile_rows_fp64(smem, row0, nr, rb, re, seg_b, lm, epi);
-      return;
-    }
-  }
-  {
-    const int lane = threadIdx.x & 31;
-    if (lane < nr && !((lm >> lane) & 1u)) {
-      PT s0 = PT(0), s1 = PT(0), s2 = PT(0), s3 = PT(0);
-      int p = rb - seg_b;
-      const int pe = re - seg_b;
-      for (; p + 4 <= pe; p += 4) {
-        s0 += smem[p];
-        s1 += smem[p + 1];
-        s2 += smem[p + 2];
-        s3 += smem[p + 3];
-      }
-      if (p < pe) s0 += smem[p];
-      if (p + 1 < pe) s1 += smem[p + 1];
-      if (p + 2 < pe) s2 += smem[p + 2];
-      epi(row0 + lane, (s0 + s1) + (s2 + s3), false);
-    }
+    epi(row0 + lane, (s0 + s1) + (s2 + s3), false);
   }
 }
-
 
 // Prefetch of the line holding *p into L1 (no register is held while it is in flight).
 __device__ __forceinline__ void prefetch_l1(const void *p) {
@@ -1020,65 +973,72 @@ __device__ __forceinline__ void walk_tile(const SideLayout &lay, const SideVals<
   if (lane >= nr - 1) re = seg_e;
   stage_segment<VT, PT, U, CP>(lay, vals, src, smem, seg_b, seg_e);
   __syncwarp();
-  tile_rows<PT>(smem, row0, nr, rb, re, seg_b, lay.long_mask[st], lay.wide_rows != 0, epi);
+  tile_rows<PT>(smem, row0, nr, rb, re, seg_b, lay.long_mask[st], epi);
   __syncwarp();
 }
 
-// GROUPED = false is the walk of layouts with tile_mult == 1 only (one tile per item, fewer
-// registers); GROUPED = true walks any layout.
+// One work item of the walk, by the whole warp.  GROUPED = false is the walk of layouts with
+// tile_mult == 1 only (one tile per item, fewer registers); GROUPED = true walks any layout.
 // pre(row) is called by the lane of each short-tile row before the tile's entries are staged,
 // so that what the row's epilogue will read can be requested while the staging round trips run.
+template <typename VT, typename PT, bool GROUPED, int U, int CP, typename Src, typename Epi,
+          typename GroupDone, typename Pre>
+__device__ __forceinline__ void walk_item(const SideLayout &lay, const SideVals<VT> vals,
+                                          const Src &src, PT *smem, const WalkScratch ws,
+                                          Epi &epi, GroupDone &gdone, const Pre &pre, int item) {
+  const int lane = threadIdx.x & 31;
+  if (item < lay.n_chunks) {
+    walk_chunk<VT, PT, CP>(lay, vals, src, ws, epi, gdone, item);
+  } else if constexpr (!GROUPED) {
+    walk_tile<VT, PT, U, CP>(lay, vals, src, smem, epi, pre, item - lay.n_chunks);
+  } else {
+    // a group of nt <= tile_mult consecutive short tiles, staged as one segment
+    const int t0 = (item - lay.n_chunks) * lay.tile_mult;
+    const int nt = min(lay.tile_mult, lay.n_short_tiles - t0);
+    for (int r = t0 * kTileRows + lane; r < min((t0 + nt) * kTileRows, lay.nrows); r += kWarp)
+      pre(r);
+    // the tiles' row starts (requested into L1 for the row sums), ends and long-row masks
+    for (int m = 1; m < nt; ++m) {
+      const int row0 = (t0 + m) * kTileRows;
+      prefetch_l1(lay.ptr_s + row0 + min(lane, lay.nrows - 1 - row0));
+    }
+    int te = 0;
+    uint32_t lmk = 0u;
+    if (lane < nt) {
+      te = lay.tile_end[t0 + lane];
+      lmk = lay.long_mask[t0 + lane];
+    }
+    const int rb0 = lay.ptr_s[t0 * kTileRows + min(lane, lay.nrows - 1 - t0 * kTileRows)];
+    const int seg_b = __shfl_sync(0xffffffffu, rb0, 0);     // 4-aligned
+    const int seg_e = __shfl_sync(0xffffffffu, te, nt - 1);
+    stage_segment<VT, PT, U, CP>(lay, vals, src, smem, seg_b, seg_e);
+    __syncwarp();
+#pragma unroll 1
+    for (int m = 0; m < nt; ++m) {
+      const int row0 = (t0 + m) * kTileRows;
+      const int nr = min(kTileRows, lay.nrows - row0);
+      const int rb = m == 0 ? rb0 : lay.ptr_s[row0 + min(lane, nr - 1)];
+      const int te_m = __shfl_sync(0xffffffffu, te, m);
+      const uint32_t lm_m = __shfl_sync(0xffffffffu, lmk, m);
+      int re = __shfl_down_sync(0xffffffffu, rb, 1);
+      if (lane >= nr - 1) re = te_m;
+      tile_rows<PT>(smem, row0, nr, rb, re, seg_b, lm_m, epi);
+    }
+    __syncwarp();
+  }
+}
+
 template <typename VT, typename PT, bool GROUPED = true, int U = kStageUnroll, int CP = 0,
           typename Src, typename Epi, typename GroupDone, typename Pre = NoPrefetch>
 __device__ __forceinline__ void walk_tiles(const SideLayout &lay, const SideVals<VT> vals,
                                            const Src &src, PT *smem, const WalkScratch ws,
                                            Epi &epi, GroupDone &gdone,
                                            const Pre &pre = Pre()) {
-  const int lane = threadIdx.x & 31;
   const int gwarp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int nwarps = gridDim.x * (blockDim.x >> 5);
   const int total = lay.total_items();
-  for (int item = gwarp; item < total; item += nwarps) {
-    if (item < lay.n_chunks) {
-      walk_chunk<VT, PT, CP>(lay, vals, src, ws, epi, gdone, item);
-    } else if constexpr (!GROUPED) {
-      walk_tile<VT, PT, U, CP>(lay, vals, src, smem, epi, pre, item - lay.n_chunks);
-    } else {
-      // a group of nt <= tile_mult consecutive short tiles, staged as one segment
-      const int t0 = (item - lay.n_chunks) * lay.tile_mult;
-      const int nt = min(lay.tile_mult, lay.n_short_tiles - t0);
-      for (int r = t0 * kTileRows + lane; r < min((t0 + nt) * kTileRows, lay.nrows); r += kWarp)
-        pre(r);
-      // the tiles' row starts (requested into L1 for the row sums), ends and long-row masks
-      for (int m = 1; m < nt; ++m) {
-        const int row0 = (t0 + m) * kTileRows;
-        prefetch_l1(lay.ptr_s + row0 + min(lane, lay.nrows - 1 - row0));
-      }
-      int te = 0;
-      uint32_t lmk = 0u;
-      if (lane < nt) {
-        te = lay.tile_end[t0 + lane];
-        lmk = lay.long_mask[t0 + lane];
-      }
-      const int rb0 = lay.ptr_s[t0 * kTileRows + min(lane, lay.nrows - 1 - t0 * kTileRows)];
-      const int seg_b = __shfl_sync(0xffffffffu, rb0, 0);     // 4-aligned
-      const int seg_e = __shfl_sync(0xffffffffu, te, nt - 1);
-      stage_segment<VT, PT, U, CP>(lay, vals, src, smem, seg_b, seg_e);
-      __syncwarp();
-#pragma unroll 1
-      for (int m = 0; m < nt; ++m) {
-        const int row0 = (t0 + m) * kTileRows;
-        const int nr = min(kTileRows, lay.nrows - row0);
-        const int rb = m == 0 ? rb0 : lay.ptr_s[row0 + min(lane, nr - 1)];
-        const int te_m = __shfl_sync(0xffffffffu, te, m);
-        const uint32_t lm_m = __shfl_sync(0xffffffffu, lmk, m);
-        int re = __shfl_down_sync(0xffffffffu, rb, 1);
-        if (lane >= nr - 1) re = te_m;
-        tile_rows<PT>(smem, row0, nr, rb, re, seg_b, lm_m, lay.wide_rows != 0, epi);
-      }
-      __syncwarp();
-    }
-  }
+  for (int item = gwarp; item < total; item += nwarps)
+    walk_item<VT, PT, GROUPED, U, CP>(lay, vals, src, smem, ws, epi, gdone, pre, item);
 }
 
 }  // namespace rh

@@ -10,10 +10,10 @@ namespace rh {
 
 // reduced cost lambda = proj onto {0} (free), [0,inf) (l finite), (-inf,0] (u finite), R
 __device__ __forceinline__ double proj_lambda(double g, double l, double u) {
-  const bool lf = isfinite(l), uf = isfinite(u);
+  const bool lf = dbl_finite(l), uf = dbl_finite(u);
   if (lf && uf) return g;
-  if (lf) return fmax(g, 0.0);
-  if (uf) return fmin(g, 0.0);
+  if (lf) return dbl_pos_part(g);
+  if (uf) return dbl_neg_part(g);
   return 0.0;
 }
 
@@ -331,7 +331,7 @@ __device__ __forceinline__ void row_epilogue(int i, double dot, const RowVecs &v
     }
   }
   double yn = yi + sigma * (qi - 2.0 * dot + kxi);
-  if (i >= f.m_eq) yn = fmax(yn, 0.0);
+  if (i >= f.m_eq) yn = dbl_pos_part(yn);
   v.yt[i] = yn;
   v.kxt[i] = dot;
   const double dy = yi - yn;
@@ -341,7 +341,7 @@ __device__ __forceinline__ void row_epilogue(int i, double dot, const RowVecs &v
   S.s[2] += ya * ya;
   if (f.check) {
     double r = (qi - dot) * v.dinv[i];
-    if (i >= f.m_eq) r = fmax(r, 0.0);
+    if (i >= f.m_eq) r = dbl_pos_part(r);
     S.s[3] += r * r;
     S.s[4] += qi * yn;
   }
@@ -366,7 +366,7 @@ __device__ __forceinline__ void col_cert_parts(int j, double d, double kv, const
                                                int s0, int m0, double *cert) {
   S.s[s0] += cj * d;
   const double du = d * v.e[j];
-  const bool lf = isfinite(lj), uf = isfinite(uj);
+  const bool lf = dbl_finite(lj), uf = dbl_finite(uj);
   if (lf) M.mx[m0] = fmax(M.mx[m0], fmax(-du, 0.0));
   if (uf) M.mx[m0 + 1] = fmax(M.mx[m0 + 1], fmax(du, 0.0));
   if (uf) S.s[s0 + 1] += fmax(kv, 0.0) * uj;
@@ -421,8 +421,8 @@ __device__ __forceinline__ void col_epilogue(int j, double dot, const ColVecs &v
     const double rd = (g - lam) * v.einv[j];
     S.s[2] += rd * rd;
     S.s[3] += cj * xtj;
-    if (lam > 0.0) S.s[4] += lj * lam;
-    else if (lam < 0.0) S.s[4] += uj * lam;
+    if (dbl_pos(lam)) S.s[4] += lj * lam;
+    else if (dbl_neg(lam)) S.s[4] += uj * lam;
     v.xout[j] = xtj;
   }
   double x0j = v.x0[j], kty0j = v.kty0[j];
@@ -447,7 +447,7 @@ __device__ __forceinline__ void col_epilogue(int j, double dot, const ColVecs &v
     kn = w * dot + (1.0 - w) * kty0j;
   }
   if (!RHO2 && f.stash) { v.x[j] = xn; v.kty[j] = kn; }
-  const double xtn = fmin(fmax(xn - tau * (cj - kn), lj), uj);
+  const double xtn = dbl_clamp(xn - tau * (cj - kn), lj, uj);
   v.xt[j] = xtn;
   const double dx = xn - xtn;
   S.s[0] += dx * dx;

@@ -1,8 +1,8 @@
 // Host plan of one side's tiled split-CSR layout, computed from the row pointers alone: which
 // rows are long, where every row's entries go, the chunks of the long rows, the staging stride,
-// how many consecutive short tiles one walk item covers, and whether the FP64 walks sum a tile's
-// longest rows warp-wide.  build_side uploads it; the C ABI
-// exposes its summary (rhpdhg_plan_layout) so the rule can be checked without a GPU.
+// how many consecutive short tiles one walk item covers, and whether its tiles are skewed.  Kernels
+// of setup.cu make the same plan in device memory (build_side); the C ABI exposes this one's summary
+// (rhpdhg_plan_layout) so the rule can be checked without a GPU.
 #pragma once
 
 #include <cstdint>
@@ -20,7 +20,7 @@ struct SidePlan {
   long long nnz_s = 0, nnz_l = 0;   // padded lengths of the short and long arrays
   long long maxseg = 0;             // longest segment of one work item's tile group
   int mult = 1;                     // short tiles per work item
-  int wide_rows = 0;                // FP64 walks sum a tile's longest rows warp-wide
+  int wide_rows = 0;                // reported: skewed tiles (wide_rows_pay in setup.cu)
   // longest segment of a work item's tile group with 1, 2 and 4 tiles per item (-1 where it
   // exceeds the staging budget): the walks the autotuner may choose instead of the rule's
   long long maxseg_mult[3] = {0, -1, -1};

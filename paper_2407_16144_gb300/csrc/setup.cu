@@ -781,16 +781,15 @@ size_t buf_drop_cache() {
   return freed;
 }
 
-// Warp-wide sums are enabled when they save at least 15% of the FP64 adds.
+// A side is reported as skewed when summing its tiles' longest rows by whole warps would save at
+// least 15% of the FP64 adds of lane-per-row sums.
 static bool wide_pays(long long plain, long long best) {
   return plain > 0 && (double)best <= 0.85 * (double)plain;
 }
 
-// The cost model of tile_rows_fp64 over all short tiles of a side: FP64 adds per warp of the
-// lane-per-row sums (4 ceil(longest / 4) per tile) against the best threshold's (c + the sum over
-// rows longer than c of ceil(len / 32) + 5, c in 8, 16, 32).  The warp-wide sums are enabled
-// when they save at least 15% of those adds (power-law sides; not sides of even row lengths,
-// where the search would only cost time).
+// That cost model over all short tiles: FP64 adds per warp of the lane-per-row sums (the longest
+// row, rounded up to 4) against the best threshold's (c + the sum over rows longer than c of
+// ceil(len / 32) + 5, c in 8, 16, 32).
 static bool wide_rows_pay(const int *hp, const std::vector<uint32_t> &mask, int nrows) {
   long long plain = 0, best = 0;
   for (int t = 0; t * kTileRows < nrows; ++t) {
