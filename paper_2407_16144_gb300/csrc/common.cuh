@@ -376,6 +376,115 @@ __device__ __forceinline__ double (*cta_red())[kMaxPartials] {
   return red;
 }
 
+// Warp sums of N slots at once (N = 1, 2 or 4): lane l returns the sum over the warp of slot
+// l / (32 / N).  While more than one slot is left, a lane keeps half of them and hands its partner
+// the other half, so 4 slots take 6 additions per lane instead of 20.  Each slot's additions are
+// those of warp_sum's tree (lanes 16, 8, 4, 2, 1 apart; an addition's operands may change places),
+// so the result has the same bits.  An FP64 addition takes 64 clocks whatever its mask, so a stage's
+// tail was mostly these trees: with it 75k entries in mixed precision 22.6 to 18.3 us an iteration.
+template <int N, class T, class Add, class Xor>
+__device__ __forceinline__ T warp_reduce_slots(T (&v)[N], Add add, Xor from_xor) {
+  static_assert(N == 1 || N == 2 || N == 4, "slots per reduction");
+  const int lane = threadIdx.x & 31;
+  int o = 16;
+#pragma unroll
+  for (int k = N; k > 1; k /= 2, o >>= 1) {
+    const bool hi = lane & o;
+#pragma unroll
+    for (int i = 0; i < k / 2; ++i) {
+      const T send = hi ? v[i] : v[i + k / 2], keep = hi ? v[i + k / 2] : v[i];
+      v[i] = add(keep, from_xor(send, o));
+    }
+  }
+  T r = v[0];
+#pragma unroll
+  for (; o > 0; o >>= 1) r = add(r, from_xor(r, o));
+  return r;
+}
+__device__ __forceinline__ double xor_f64(double v, int o) {
+  return __shfl_xor_sync(0xffffffffu, v, o);
+}
+template <bool EXACT>
+__device__ __forceinline__ DF xor_df(DF v, int o) {
+  DF w;
+  w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
+  w.lo = EXACT ? __shfl_xor_sync(0xffffffffu, v.lo, o) : 0.f;
+  return w;
+}
+
+// The warp's sums of the slots in smask and maxima of the slots in mmask of an accumulator, written
+// to dst[slot] (sums, then maxima at NS; the first ND sums double-floats, bit-packed).  Slots in
+// prewarp hold, in lane 0, a value already summed over the warp (FP64 slots only).
+template <int NS, int NM, int ND, bool EXACT, class A>
+__device__ __forceinline__ void warp_reduce_to(A &a, unsigned smask, unsigned mmask,
+                                               unsigned prewarp, double *dst) {
+  const int lane = threadIdx.x & 31;
+  if constexpr (ND > 0) {
+    static_assert(ND <= 4, "one group of packed slots");
+    constexpr int N = ND == 1 ? 1 : ND == 2 ? 2 : 4;
+    if (smask & ((1u << ND) - 1u)) {
+      DF v[N];
+#pragma unroll
+      for (int i = 0; i < N; ++i) v[i] = i < ND ? a.d[i < ND ? i : 0] : DF{0.f, 0.f};
+      const DF r = warp_reduce_slots<N>(
+          v, [](DF x, DF y) { return dfx_add<EXACT>(x, y); },
+          [](DF x, int o) { return xor_df<EXACT>(x, o); });
+      const int i = lane / (32 / N);
+      if (lane % (32 / N) == 0 && i < ND && ((smask >> i) & 1u)) dst[i] = df_pack(r);
+    }
+  }
+#pragma unroll
+  for (int g = ND; g < NS; g += 4) {
+    const unsigned mine = (smask >> g) & 0xfu & ((1u << (NS - g < 4 ? NS - g : 4)) - 1u);
+    if (!mine) continue;
+    double v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = g + i < NS && ((mine >> i) & 1u) ? a.s[g + i < NS ? g + i : 0] : 0.0;
+    const unsigned pre = (prewarp >> g) & mine;
+    if (pre) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if ((mine >> i) & 1u) {
+          const double r = ((pre >> i) & 1u) ? v[i] : warp_sum(v[i]);
+          if (lane == 0) dst[g + i] = r;
+        }
+      continue;
+    }
+    double r;
+    int i;
+    if (mine & 0xcu) {
+      r = warp_reduce_slots<4>(v, [](double x, double y) { return x + y; }, xor_f64);
+      i = lane / 8;
+      if (lane % 8) i = 4;
+    } else {
+      double w[2] = {v[0], v[1]};
+      r = warp_reduce_slots<2>(w, [](double x, double y) { return x + y; }, xor_f64);
+      i = lane / 16;
+      if (lane % 16) i = 4;
+    }
+    if (i < 4 && ((mine >> i) & 1u)) dst[g + i] = r;
+  }
+#pragma unroll
+  for (int i = 0; i < NM; ++i) {
+    if (!((mmask >> i) & 1u)) continue;
+    const double v = warp_max(a.mx[i]);
+    if (lane == 0) dst[NS + i] = v;
+  }
+}
+
+// Thread i of the first warp: slot i's value over the CTA's nw warps (rows of red), in warp order.
+template <int NS, int NM, int ND, bool EXACT>
+__device__ __forceinline__ double cta_slot(const double (*red)[kMaxPartials], int i, int nw) {
+  double v = red[0][i];
+  if (i < ND) {
+    DF d = df_unpack(v);
+    for (int w = 1; w < nw; ++w) d = dfx_add<EXACT>(d, df_unpack(red[w][i]));
+    return df_pack(d);
+  }
+  for (int w = 1; w < nw; ++w) v = i < NS ? v + red[w][i] : fmax(v, red[w][i]);
+  return v;
+}
+
 // Reduce Acc over the CTA (deterministic: fixed shuffle tree, warps summed in index order) and
 // write the CTA's partials to part[blockIdx.x * kMaxPartials + slot] (double-float slots
 // bit-packed).  Only the slots set in smask (sums) and mmask (maxima) are reduced and written;
@@ -389,47 +498,16 @@ __device__ bool cta_reduce_and_ticket(Acc<NS, NM, ND, EXACT> &a, unsigned smask,
   __shared__ bool last;
   static_assert(NS + NM <= kMaxPartials, "too many partial slots");
   static_assert(ND <= NS, "double-float slots are sums");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int i = 0; i < NS; ++i) {
-    if (!((smask >> i) & 1u)) continue;
-    if (i < ND) {
-      const DF v = dfx_warp_sum<EXACT>(a.d[i < ND ? i : 0]);
-      if (lane == 0) red[warp][i] = df_pack(v);
-    } else {
-      const double v = ((prewarp >> i) & 1u) ? a.s[i] : warp_sum(a.s[i]);
-      if (lane == 0) red[warp][i] = v;
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < NM; ++i) {
-    if (!((mmask >> i) & 1u)) continue;
-    const double v = warp_max(a.mx[i]);
-    if (lane == 0) red[warp][NS + i] = v;
-  }
+  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  warp_reduce_to<NS, NM, ND, EXACT>(a, smask, mmask, prewarp, red[warp]);
   __syncthreads();
+  if (warp == 0) {
+    const int i = threadIdx.x;
+    if (((smask | (mmask << NS)) >> i) & 1u)
+      part[(size_t)blockIdx.x * kMaxPartials + i] = cta_slot<NS, NM, ND, EXACT>(red, i, nw);
+    __syncwarp();              // before lane 0's fence
+  }
   if (threadIdx.x == 0) {
-    double *dst = part + (size_t)blockIdx.x * kMaxPartials;
-#pragma unroll
-    for (int i = 0; i < NS; ++i) {
-      if (!((smask >> i) & 1u)) continue;
-      if (i < ND) {
-        DF v = df_unpack(red[0][i]);
-        for (int w = 1; w < nw; ++w) v = dfx_add<EXACT>(v, df_unpack(red[w][i]));
-        dst[i] = df_pack(v);
-      } else {
-        double v = red[0][i];
-        for (int w = 1; w < nw; ++w) v += red[w][i];
-        dst[i] = v;
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < NM; ++i) {
-      if (!((mmask >> i) & 1u)) continue;
-      double v = red[0][NS + i];
-      for (int w = 1; w < nw; ++w) v = fmax(v, red[w][NS + i]);
-      dst[NS + i] = v;
-    }
     if constexpr (TICKET) {
       __threadfence();
       const unsigned int tk = atomicAdd(ticket, 1u);
@@ -460,24 +538,13 @@ __device__ void cta_reduce_store(Acc<NS, NM, ND, EXACT> &a, unsigned smask, unsi
 template <int NS, int ND, bool EXACT>
 __device__ __forceinline__ void store_group(Acc<NS, 0, ND, EXACT> &al, unsigned smask,
                                             double *gpart, int grp) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int i = 0; i < NS; ++i) {
-    if (!((smask >> i) & 1u)) continue;
-    if (i < ND) {
-      const DF v = dfx_warp_sum<EXACT>(al.d[i < ND ? i : 0]);
-      if (lane == 0) gpart[(size_t)grp * kMaxPartials + i] = df_pack(v);
-    } else {
-      const double v = warp_sum(al.s[i]);
-      if (lane == 0) gpart[(size_t)grp * kMaxPartials + i] = v;
-    }
-  }
+  warp_reduce_to<NS, 0, ND, EXACT>(al, smask, 0u, 0u, gpart + (size_t)grp * kMaxPartials);
   al.zero();
 }
 
 // In the last CTA: reduce the grid's partials in block order, then the long-row groups'
 // partials in group order, for the slots in the masks (others return 0; the first ND sums are
-// double-floats, returned as hi + lo).  out[i] valid in all threads.
+// double-floats, returned as hi + lo).  out[i] valid in the first warp.
 //
 // Thread t sums blocks t, t + blockDim, ... of each slot in that order, then groups t,
 // t + blockDim, ...; each warp reduces its lanes with a fixed shuffle tree and the warps' results
@@ -543,30 +610,24 @@ __device__ void grid_finish(const double *part, double *out, unsigned smask, uns
       take(i, __ldcg(src + i));
     }
   }
+  Acc<NS, NM, ND, EXACT> t;
 #pragma unroll
-  for (int i = 0; i < NS + NM; ++i) {
-    if (!((all >> i) & 1u)) continue;
-    if (i < ND) {
-      const DF r = dfx_warp_sum<EXACT>(vd[i < ND ? i : 0]);
-      if (lane == 0) red[warp][i] = df_pack(r);
-    } else {
-      const double r = (i < NS) ? warp_sum(v[i]) : warp_max(v[i]);
-      if (lane == 0) red[warp][i] = r;
-    }
-  }
+  for (int i = 0; i < NS; ++i) t.s[i] = v[i];
+#pragma unroll
+  for (int i = 0; i < NM; ++i) t.mx[i] = v[NS + i];
+#pragma unroll
+  for (int i = 0; i < ND; ++i) t.d[i] = vd[i];
+  warp_reduce_to<NS, NM, ND, EXACT>(t, smask, mmask, 0u, red[warp]);
   __syncthreads();
-#pragma unroll
-  for (int i = 0; i < NS + NM; ++i) {
-    if (!((all >> i) & 1u)) { out[i] = 0.0; continue; }
-    if (i < ND) {
-      DF r = df_unpack(red[0][i]);
-      for (int w = 1; w < nw; ++w) r = dfx_add<EXACT>(r, df_unpack(red[w][i]));
-      out[i] = df_value(r);
-    } else {
-      double r = red[0][i];
-      for (int w = 1; w < nw; ++w) r = (i < NS) ? r + red[w][i] : fmax(r, red[w][i]);
-      out[i] = r;
+  if (warp == 0) {
+    double r = 0.0;
+    if ((all >> lane) & 1u) {
+      r = cta_slot<NS, NM, ND, EXACT>(red, lane, nw);
+      if (lane < ND) r = df_value(df_unpack(r));
     }
+#pragma unroll
+    for (int i = 0; i < NS + NM; ++i)
+      out[i] = ((all >> i) & 1u) ? __shfl_sync(0xffffffffu, r, i) : 0.0;
   }
   __syncthreads();
 }
@@ -577,7 +638,7 @@ __device__ void grid_finish(const double *part, double *out, unsigned smask, uns
 // row reduction's; dcol_finish adds them, any further rows and the column's long-row groups in
 // the order grid_finish uses (a thread's rows in index order, then its groups; lanes by the
 // shuffle tree; warps in index order), and returns the sums (the first ND double-floats) in
-// every thread.
+// the first warp.
 constexpr int kDcolPre = 4;
 constexpr int kDcolBatch = 6;
 struct DcolPre {
@@ -633,28 +694,21 @@ __device__ void dcol_finish(const DeferredCol &dc, const DcolPre &pre, double *o
     take(0, __ldcg(src));
     take(1, __ldcg(src + 1));
   }
+  Acc<2, 0, ND, EXACT> t;
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    if (i < ND) {
-      const DF r = dfx_warp_sum<EXACT>(vd[i]);
-      if (lane == 0) red[warp][i] = df_pack(r);
-    } else {
-      const double r = warp_sum(v[i]);
-      if (lane == 0) red[warp][i] = r;
-    }
-  }
+  for (int i = 0; i < 2; ++i) t.s[i] = v[i];
+#pragma unroll
+  for (int i = 0; i < ND; ++i) t.d[i] = vd[i];
+  warp_reduce_to<2, 0, ND, EXACT>(t, 0x3u, 0u, 0u, red[warp]);
   __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    if (i < ND) {
-      DF r = df_unpack(red[0][i]);
-      for (int w = 1; w < nw; ++w) r = dfx_add<EXACT>(r, df_unpack(red[w][i]));
-      out[i] = df_value(r);
-    } else {
-      double r = red[0][i];
-      for (int w = 1; w < nw; ++w) r += red[w][i];
-      out[i] = r;
+  if (warp == 0) {
+    double r = 0.0;
+    if (lane < 2) {
+      r = cta_slot<2, 0, ND, EXACT>(red, lane, nw);
+      if (lane < ND) r = df_value(df_unpack(r));
     }
+    out[0] = __shfl_sync(0xffffffffu, r, 0);
+    out[1] = __shfl_sync(0xffffffffu, r, 1);
   }
   __syncthreads();
 }
@@ -808,92 +862,36 @@ __device__ __forceinline__ void walk_chunk(const SideLayout &lay, const SideVals
   }
 }
 
-// Row sums of one warp's staged segment s[0, len), balanced over the lanes: returns, in lane r, the
-// sum of s[b, e) (b, e: that lane's row, 0 <= b <= e <= len; rows in lane order without overlap,
-// so the rows that are not empty tile [b of the first, e of the last)).  The segment's contents are
-// consumed.
-//
-// What bounds it is the FP64 pipe, which is narrow on this part and issues a warp's add as slowly
-// for one active lane as for 32: one lane per row costs the longest row's adds.  Here every lane
-// adds an equal run of L consecutive entries (L odd: no shared-memory bank conflicts), writing its
-// running sum over the last entry of every row, and of the run, that it completes; lane r then adds
-// the one or few partial sums of its row, in entry order.  That is L + (runs a row spans) adds for
-// the warp.  Where no row is longer than that, one lane per row is kept.  Measured with the integer
-// comparisons above, FP64 iterations against lane-per-row sums (or, on skewed sides, sums of the
-// longest rows by the whole warp): 2.5M entries with power-law columns 112 to 93 us, flow LP of 30M
-// entries 797 to 703 us, 150k even entries 36 to 34 us.
-template <typename PT>
-__device__ __forceinline__ PT balanced_row_sum(PT *s, int len, int b, int e) {
-  const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  const int mx = (int)__reduce_max_sync(full, (unsigned)(e - b));
-  const int L = ((len + kWarp - 1) / kWarp) | 1;
-  if (mx <= L + (mx + L - 2) / L) {
-    PT t = PT(0);
-#pragma unroll 4
-    for (int p = b; p < e; ++p) t += s[p];
-    return t;
-  }
-  // the row that holds this lane's first entry: the number of rows that end at or before it
-  const int start = lane * L, stop = min(start + L, len);
-  int r = 0;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-    if (__shfl_sync(full, e, r + o - 1) <= start) r += o;
-  const unsigned some = __ballot_sync(full, e > b);
-  int end = __shfl_sync(full, e, r);
-  PT acc = PT(0);
-#pragma unroll 4
-  for (int i = 0; i < L; ++i) {
-    const int p = start + i;
-    const bool in = p < stop;
-    if (in) acc += s[p];
-    const bool done = p + 1 == end;
-    if (in && (done || i == L - 1)) s[p] = acc;
-    if (done) {
-      acc = PT(0);
-      const unsigned rest = some & ~((2u << r) - 1u);   // the next row that is not empty
-      r = rest ? __ffs((int)rest) - 1 : r;
-    }
-    end = __shfl_sync(full, e, r);
-  }
-  __syncwarp();
-  PT t = PT(0);
-  if (e > b) {
-    // run of an entry by a multiplication: exact for entries below 1056 and L up to 33
-    static_assert(kSegBudget <= 1024, "entries of a staged segment");
-    const unsigned inv = (65536u + (unsigned)L - 1u) / (unsigned)L;
-    int c = (int)(((unsigned)b * inv) >> 16);
-    const int c1 = (int)(((unsigned)(e - 1) * inv) >> 16);
-    t = s[min((c + 1) * L, e) - 1];
-    while (c < c1) {
-      ++c;
-      t += s[min((c + 1) * L, e) - 1];
-    }
-  }
-  return t;
-}
-
 // Sums the rows of a short tile from the staged products smem[0, ...) (staged from seg_b on) and
-// runs their epilogues, lane r row r (rows marked long in lm are skipped).  FP64 tiles balance the
-// additions over the lanes (balanced_row_sum); FP32 tiles, whose pipe is wide, sum lane per row
-// with four interleaved accumulators, each lane going on to its epilogue as soon as its row is
-// summed, so that its loads overlap the other lanes' sums.
+// runs their epilogues, lane r row r (rows marked long in lm are skipped), each lane going on to its
+// epilogue as soon as its row is summed, so that its loads overlap the other lanes' sums.
+//
+// FP64: the pipe is narrow on this part; an instruction takes 64 clocks of its scheduler with one
+// active lane or 32, so one lane per row costs the longest row's additions.  The groups of four
+// that stage_segment adds up (one fused multiply-add per entry, every lane busy) leave a quarter
+// of them.  Per FP64 iteration, with warp_reduce_slots, against runs of entries balanced over the
+// lanes and a tree per slot: 2.5M entries with power-law columns 93 to 75 us, flow LP of 30M entries
+// 702 to 621 us, 150k even entries 32 to 21 us.  FP32: four interleaved accumulators.
 template <typename PT, typename Epi>
-__device__ __forceinline__ void tile_rows(PT *smem, int row0, int nr, int rb, int re,
+__device__ __forceinline__ void tile_rows(const PT *smem, int row0, int nr, int rb, int re,
                                           int seg_b, uint32_t lm, Epi &epi) {
   const int lane = threadIdx.x & 31;
-  const bool act = lane < nr && !((lm >> lane) & 1u);
+  if (lane >= nr || ((lm >> lane) & 1u)) return;
+  int p = rb - seg_b;
+  const int pe = re - seg_b;
   if constexpr (sizeof(PT) == sizeof(double)) {
-    const int tb = __shfl_sync(0xffffffffu, rb, 0), te = __shfl_sync(0xffffffffu, re, nr - 1);
-    // (a long row's short range is empty; lanes past the last row take an empty one at the end)
-    const int b = lane < nr ? rb - tb : te - tb, e = lane < nr ? re - tb : te - tb;
-    const PT dot = balanced_row_sum(smem + (tb - seg_b), te - tb, b, e);
-    if (act) epi(row0 + lane, dot, false);
-  } else if (act) {
+    PT dot = PT(0);
+    if (p < pe) {
+      int q = p | 3;                         // the group's last entry
+      dot = smem[min(q, pe - 1)];
+      while (q < pe - 1) {
+        q += 4;
+        dot += smem[min(q, pe - 1)];
+      }
+    }
+    epi(row0 + lane, dot, false);
+  } else {
     PT s0 = PT(0), s1 = PT(0), s2 = PT(0), s3 = PT(0);
-    int p = rb - seg_b;
-    const int pe = re - seg_b;
     for (; p + 4 <= pe; p += 4) {
       s0 += smem[p];
       s1 += smem[p + 1];
@@ -919,10 +917,13 @@ struct NoPrefetch {
 
 // Stage the products of the segment [seg_b, seg_e) (seg_b 4-aligned) in smem[0, ...): lane
 // handles 4-entry groups g = lane, lane + 32, ..., U at a time (more loads in flight per round,
-// more registers).
+// more registers).  FP32 products are staged one by one.  FP64 products are added up within their
+// group of four, up to a row's end (a set bit of ends, see row_ends): smem[p] holds, where entry p
+// ends its row or its group, the sum of the row's entries in the group, and nothing elsewhere.
 template <typename VT, typename PT, int U, int CP, typename Src>
 __device__ __forceinline__ void stage_segment(const SideLayout &lay, const SideVals<VT> vals,
-                                              const Src &src, PT *smem, int seg_b, int seg_e) {
+                                              const Src &src, PT *smem, int seg_b, int seg_e,
+                                              const unsigned *ends) {
   const int lane = threadIdx.x & 31;
   const int nvec = (seg_e - seg_b + 3) >> 2;             // groups of 4 entries
   constexpr int kU = U;
@@ -949,11 +950,39 @@ __device__ __forceinline__ void stage_segment(const SideLayout &lay, const SideV
     for (int u = 0; u < kU; ++u) {
       const int g = g0 + u * kWarp + lane;
       if (g < nvec) {
+        if constexpr (sizeof(PT) == sizeof(double)) {
+          const unsigned end = ends[g >> 3] >> (4 * (g & 7));
+          PT acc = vv[u].v[0] * x[u][0];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) smem[4 * g + e] = PT(vv[u].v[e]) * x[u][e];
+          for (int e = 1; e < 4; ++e) {
+            const bool done = (end >> (e - 1)) & 1u;
+            if (done) smem[4 * g + e - 1] = acc;
+            acc = fma(vv[u].v[e], x[u][e], done ? PT(0) : acc);
+          }
+          smem[4 * g + 3] = acc;
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) smem[4 * g + e] = PT(vv[u].v[e]) * x[u][e];
+        }
       }
     }
   }
+}
+
+// The row ends of the segment that starts at seg_b, a bit per entry in 32 words of shared memory
+// of the warp, for FP64 stagings: cleared, then set by each lane for its row [rb, re) of each of
+// the segment's tiles.
+__device__ __forceinline__ unsigned *row_ends_clear() {
+  __shared__ unsigned words[kMaxBlockWarps][kWarp];
+  static_assert(kSegBudget <= 32 * kWarp, "a bit per entry of a staged segment");
+  unsigned *w = words[threadIdx.x >> 5];
+  w[threadIdx.x & 31] = 0u;
+  __syncwarp();
+  return w;
+}
+__device__ __forceinline__ void row_end(unsigned *ends, int seg_b, int rb, int re) {
+  const int p = re - 1 - seg_b;
+  if (re > rb) atomicOr(ends + (p >> 5), 1u << (p & 31));
 }
 
 // One short tile st of walk_tiles (tile_mult == 1): stage its segment, then lane r sums row r
@@ -971,7 +1000,13 @@ __device__ __forceinline__ void walk_tile(const SideLayout &lay, const SideVals<
   const int seg_b = __shfl_sync(0xffffffffu, rb, 0);     // 4-aligned
   int re = __shfl_down_sync(0xffffffffu, rb, 1);
   if (lane >= nr - 1) re = seg_e;
-  stage_segment<VT, PT, U, CP>(lay, vals, src, smem, seg_b, seg_e);
+  unsigned *ends = nullptr;
+  if constexpr (sizeof(PT) == sizeof(double)) {
+    ends = row_ends_clear();
+    if (lane < nr) row_end(ends, seg_b, rb, re);
+    __syncwarp();
+  }
+  stage_segment<VT, PT, U, CP>(lay, vals, src, smem, seg_b, seg_e, ends);
   __syncwarp();
   tile_rows<PT>(smem, row0, nr, rb, re, seg_b, lay.long_mask[st], epi);
   __syncwarp();
@@ -1011,7 +1046,21 @@ __device__ __forceinline__ void walk_item(const SideLayout &lay, const SideVals<
     const int rb0 = lay.ptr_s[t0 * kTileRows + min(lane, lay.nrows - 1 - t0 * kTileRows)];
     const int seg_b = __shfl_sync(0xffffffffu, rb0, 0);     // 4-aligned
     const int seg_e = __shfl_sync(0xffffffffu, te, nt - 1);
-    stage_segment<VT, PT, U, CP>(lay, vals, src, smem, seg_b, seg_e);
+    unsigned *ends = nullptr;
+    if constexpr (sizeof(PT) == sizeof(double)) {
+      ends = row_ends_clear();
+      for (int m = 0; m < nt; ++m) {
+        const int row0 = (t0 + m) * kTileRows;
+        const int nr = min(kTileRows, lay.nrows - row0);
+        const int rb = lay.ptr_s[row0 + min(lane, nr - 1)];
+        const int te_m = __shfl_sync(0xffffffffu, te, m);
+        int re = __shfl_down_sync(0xffffffffu, rb, 1);
+        if (lane >= nr - 1) re = te_m;
+        if (lane < nr) row_end(ends, seg_b, rb, re);
+      }
+      __syncwarp();
+    }
+    stage_segment<VT, PT, U, CP>(lay, vals, src, smem, seg_b, seg_e, ends);
     __syncwarp();
 #pragma unroll 1
     for (int m = 0; m < nt; ++m) {

@@ -44,6 +44,69 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
   return r;   // valid in thread 0
 }
 
+// Row sums of one warp's staged segment s[0, len), balanced over the lanes: returns, in lane r, the
+// sum of s[b, e) (b, e: that lane's row, 0 <= b <= e <= len; rows in lane order without overlap,
+// so the rows that are not empty tile [b of the first, e of the last)).  The segment's contents are
+// consumed.
+//
+// What bounds it is the FP64 pipe, which is narrow on this part and issues a warp's add as slowly
+// for one active lane as for 32: one lane per row costs the longest row's adds.  Here every lane
+// adds an equal run of L consecutive entries (L odd: no shared-memory bank conflicts), writing its
+// running sum over the last entry of every row, and of the run, that it completes; lane r then adds
+// the one or few partial sums of its row, in entry order.  That is L + (runs a row spans) adds for
+// the warp.  Where no row is longer than that, one lane per row is kept.
+template <typename PT>
+__device__ __forceinline__ PT balanced_row_sum(PT *s, int len, int b, int e) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int mx = (int)__reduce_max_sync(full, (unsigned)(e - b));
+  const int L = ((len + kWarp - 1) / kWarp) | 1;
+  if (mx <= L + (mx + L - 2) / L) {
+    PT t = PT(0);
+#pragma unroll 4
+    for (int p = b; p < e; ++p) t += s[p];
+    return t;
+  }
+  // the row that holds this lane's first entry: the number of rows that end at or before it
+  const int start = lane * L, stop = min(start + L, len);
+  int r = 0;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    if (__shfl_sync(full, e, r + o - 1) <= start) r += o;
+  const unsigned some = __ballot_sync(full, e > b);
+  int end = __shfl_sync(full, e, r);
+  PT acc = PT(0);
+#pragma unroll 4
+  for (int i = 0; i < L; ++i) {
+    const int p = start + i;
+    const bool in = p < stop;
+    if (in) acc += s[p];
+    const bool done = p + 1 == end;
+    if (in && (done || i == L - 1)) s[p] = acc;
+    if (done) {
+      acc = PT(0);
+      const unsigned rest = some & ~((2u << r) - 1u);   // the next row that is not empty
+      r = rest ? __ffs((int)rest) - 1 : r;
+    }
+    end = __shfl_sync(full, e, r);
+  }
+  __syncwarp();
+  PT t = PT(0);
+  if (e > b) {
+    // run of an entry by a multiplication: exact for entries below 1056 and L up to 33
+    static_assert(kSegBudget <= 1024, "entries of a staged segment");
+    const unsigned inv = (65536u + (unsigned)L - 1u) / (unsigned)L;
+    int c = (int)(((unsigned)b * inv) >> 16);
+    const int c1 = (int)(((unsigned)(e - 1) * inv) >> 16);
+    t = s[min((c + 1) * L, e) - 1];
+    while (c < c1) {
+      ++c;
+      t += s[min((c + 1) * L, e) - 1];
+    }
+  }
+  return t;
+}
+
 // One warp takes 32 consecutive rows: their entries are read as one contiguous segment, kKktStage at
 // a time, every lane on consecutive entries (one thread per row read 12 bytes here and 12 bytes
 // 200 bytes further on).  Each entry finds its row among the 32 row ends by a search in shuffles,
