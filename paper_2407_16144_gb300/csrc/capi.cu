@@ -74,6 +74,7 @@ struct rhpdhg_handle {
   ColVecs cv{};
   int grid_row = 1, grid_col = 1, smem_row = 0, smem_col = 0;
   int grid_row1 = 1, grid_col1 = 1;   // restart-mode mixed kernels: at most one resident wave
+  bool both_row = false, both_col = false;   // mixed: one kernel per stage (see k_row_iter_mx)
   int col_rows_last = 1;              // CTA rows the last column launch wrote (see DeferredCol)
   double eta = 1.0, omega0 = 1.0, sigma_max = 0.0;
 
@@ -232,6 +233,15 @@ void set_geometry(rhpdhg_handle *h, const SideShape &r, const SideShape &c) {
     const int bc = iter_mx_restart_blocks_per_sm(h->smem_col, false, wc * kWarp);
     h->grid_row1 = std::max(1, std::min(h->grid_row, h->sm_count * std::max(br, 1)));
     h->grid_col1 = std::max(1, std::min(h->grid_col, h->sm_count * std::max(bc, 1)));
+    // one kernel per stage where its CTAs are all resident (then grid_row1 = grid_row too, and the
+    // restart iterations' sums are added in the same order)
+    auto resident = [&](bool row, const SideLayout &l, int smem, int grid, int grid1) {
+      return !h->ic.bf16 && !h->ic.df_sums && grid1 == grid &&
+             grid <= h->sm_count *
+                         iter_mx_both_blocks_per_sm(smem, row, l.walk, l.cta_warps * kWarp);
+    };
+    h->both_row = resident(true, lr, h->smem_row, h->grid_row, h->grid_row1);
+    h->both_col = resident(false, lc, h->smem_col, h->grid_col, h->grid_col1);
   } else {
     h->grid_row = tile_grid(lr, h->sm_count,
                             capped(row_iter_blocks_per_sm(h->smem_row, wr * kWarp), r.cap));
@@ -262,7 +272,7 @@ void launch_row(rhpdhg_handle *h) {
   dc.ngroups = h->cols.lay.n_long_tiles;
   if (h->mixed)
     launch_row_iter_mx(h->st, h->rows, h->rvm, h->dxt, h->dxt64, h->x0, h->ctl, h->part_row,
-                       h->ic, h->grid_row, h->grid_row1, h->smem_row, dc);
+                       h->ic, h->grid_row, h->grid_row1, h->smem_row, h->both_row, dc);
   else
     launch_row_iter(h->st, h->rows, h->xt, h->rv, h->ctl, h->part_row, h->ic, h->grid_row,
                     h->smem_row, dc);
@@ -272,10 +282,15 @@ void launch_col(rhpdhg_handle *h, int phase) {
   h->col_rows_last = h->grid_col;   // a deferring (ordinary) column launch has grid_col CTAs
   if (h->mixed)
     launch_col_iter_mx(h->st, h->cols, h->cvm, h->dyt, h->dyt64, h->y0, h->ctl, h->part_col,
-                       h->ic, h->grid_col, h->grid_col1, h->smem_col, phase);
+                       h->ic, h->grid_col, h->grid_col1, h->smem_col, h->both_col, phase);
   else
     launch_col_iter(h->st, h->cols, h->yt, h->cv, h->ctl, h->part_col, h->ic, h->grid_col,
                     h->smem_col, phase);
+}
+
+// Kernels of one iteration.
+long long launches_per_iter(const rhpdhg_handle *h) {
+  return h->mixed ? 4 - (h->both_row ? 1 : 0) - (h->both_col ? 1 : 0) : 2;
 }
 
 void launch_iteration(rhpdhg_handle *h) {
@@ -594,7 +609,7 @@ void drive(rhpdhg_handle *h) {
         }
         cudaEventRecord(ev[g], h->st);
         ++launched;
-        h->launches += (h->mixed ? 4LL : 2LL) * chunk;
+        h->launches += launches_per_iter(h) * chunk;
       }
       if (done >= launched) break;
       const int g = (int)(done & 1);
@@ -966,7 +981,7 @@ int rhpdhg_create(const rhpdhg_problem *lp, const rhpdhg_params *params, void *c
     else fill(st, n, 1.0 / std::sqrt((double)n), (double *)v);
     const double *scale = nullptr;       // v is already normalised
     for (int it = 0; it < P.power_iters; ++it) {
-      side_spmv_pw(st, h->rows, lowp, v, scale, um, pp, tk, ss + 2, gr);
+      side_spmv_pw(st, h->rows, lowp, v, scale, um, pp, tk, nullptr, gr);
       side_spmv_pw(st, h->cols, lowp, um, nullptr, w, pp, tk, ss + 4, gc);
       std::swap(v, w);
       scale = ss + 5;                    // 1 / ||K^T K^ v||

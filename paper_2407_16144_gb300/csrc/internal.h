@@ -137,7 +137,8 @@ void side_spmv(cudaStream_t st, const SideStore &side, const double *src, double
 // Power-iteration product: out = side * (src * in_scale[0]) and ss = (||out||^2, 1/||out||);
 // lowp 0: FP64 vectors, values, products and sums; 1 / 2: FP32 vectors and the side's FP32 / BF16
 // values with FP32 products and row sums (mixed-precision handles); the norm is an FP64 sum in
-// every case.  part holds grid * kMaxPartials doubles, ticket a zeroed counter.
+// every case.  part holds grid * kMaxPartials doubles, ticket a zeroed counter; ss NULL: the norm
+// is not wanted and the grid reduction is left out.
 void side_spmv_pw(cudaStream_t st, const SideStore &side, int lowp, const void *src,
                   const double *in_scale, void *out, double *part, unsigned int *ticket,
                   double *ss, int grid);
@@ -176,17 +177,20 @@ cudaError_t kkt_eval_with_scratch(const rhpdhg_problem *lp, const double *x, con
                                   double *out, bool *bad_index);
 
 // ---- mixed-precision iteration (iterate_mx.cu) -------------------------------------------------
-// grid: CTAs of the ordinary kernel; grid1: CTAs of the restart-mode kernel (at most one wave)
+// grid: CTAs of the ordinary kernel; grid1: CTAs of the restart-mode kernel (at most one wave);
+// both: one kernel of grid CTAs takes both kinds of iteration (FP32 values and sums only)
 void launch_row_iter_mx(cudaStream_t st, const SideStore &side, const RowVecsMx &v,
                         const float *dxt, const double *dxt64, const double *x0, Ctl *ctl,
                         double *part, const IterConsts &ic, int grid, int grid1, int smem,
-                        const DeferredCol &dc);
+                        bool both, const DeferredCol &dc);
 void launch_col_iter_mx(cudaStream_t st, const SideStore &side, const ColVecsMx &v,
                         const float *dyt, const double *dyt64, const double *y0, Ctl *ctl,
                         double *part, const IterConsts &ic, int grid, int grid1, int smem,
-                        int phase);
+                        bool both, int phase);
 // Resident CTAs per SM of the restart-mode mixed kernels of one side (FP64 staging smem).
 int iter_mx_restart_blocks_per_sm(int smem, bool row, int threads);
+// The same of the kernels that take both kinds of iteration, in one walk instantiation.
+int iter_mx_both_blocks_per_sm(int smem, bool row, int walk, int threads);
 void launch_unscale_mx(cudaStream_t st, int n, int m, const double *e, const double *xs,
                        const double *d, const double *y0, const float *dyt, double *xo,
                        double *yo, double *yt64);

@@ -51,21 +51,19 @@ constexpr int col_df_slots() { return MODE == 0 ? 2 : 0; }
 // warps per SM), the wide walk 80 (96 with double-float sums), the restart kernels (MODE 1) 128.
 // The CTA width is chosen at launch (up to kMaxBlockThreads).
 __host__ __device__ constexpr int mx_max_regs(int mode, int walk, int dfs) {
-  return mode == 1 ? 128 : (walk == kWalkWide ? (dfs ? 96 : 80) : 64);
+  return mode >= 1 ? 128 : (walk == kWalkWide ? (dfs ? 96 : 80) : 64);
 }
 
-// MODE 0 runs the ordinary (FP32) iterations and returns at once when a restart is pending;
-// MODE 1 runs only the restart iterations (FP64 walks) and returns at once otherwise.  Both are
-// launched every iteration; splitting them keeps the register footprint of the FP32 kernel small.
+// MODE 0 is the ordinary (FP32) iteration and returns at once when a restart is pending; MODE 1 is
+// the restart iteration (FP64 walks) and returns at once otherwise.
 // CP: the matrix stream's cache policy of the ordinary kernels' walk (see Vec4 in common.cuh).
-template <int RHO2, int MODE, int WALK, int DFS, int LP, int CP = 0>
-__global__ void __maxnreg__(mx_max_regs(MODE, WALK, DFS))
-k_row_iter_mx(SideLayout lay, SideVals<double> v64, SideVals<LowT<LP>> v32, WalkScratch wa,
-              WalkScratch wb, RowVecsMx v, const float *__restrict__ dxt,
-              const double *__restrict__ dxt64, const double *__restrict__ x0, Ctl *ctl,
-              double *part, IterConsts ic, DeferredCol dc) {
-  extern __shared__ double smem[];
-  if (ctl->status != kRunning) return;
+template <int RHO2, int MODE, int WALK, int DFS, int LP, int CP>
+__device__ __forceinline__ void
+row_iter_mx(double *smem, const SideLayout &lay, const SideVals<double> v64,
+            const SideVals<LowT<LP>> v32, const WalkScratch wa, const WalkScratch wb,
+            const RowVecsMx &v, const float *__restrict__ dxt, const double *__restrict__ dxt64,
+            const double *__restrict__ x0, Ctl *ctl, double *part, const IterConsts &ic,
+            const DeferredCol &dc) {
   // stage 1 here: the preceding ordinary column stage deferred its reduction (col_defers); this
   // iteration is the one after it (an ordinary column stage leaves no restart pending)
   const int stage = ctl->stage;
@@ -156,15 +154,41 @@ k_row_iter_mx(SideLayout lay, SideVals<double> v64, SideVals<LowT<LP>> v32, Walk
   }
 }
 
-// MODE 0: ordinary iterations (no pending restart, not a restart point); MODE 1: the rest.
+// Where every CTA of a stage is resident at once in the restart kernel's registers, one kernel
+// (MODE 2) takes both kinds of iteration.  Elsewhere the two are launched one after the other in
+// every iteration, which keeps the register footprint of the ordinary kernel small and its
+// residency high; a launch that returns at entry costs about 1.3 us.  75k entries, 640 iterations
+// with create and free: 16.2 to 14.3 ms (with the power iteration's unread norms left out).
 template <int RHO2, int MODE, int WALK, int DFS, int LP, int CP = 0>
 __global__ void __maxnreg__(mx_max_regs(MODE, WALK, DFS))
-k_col_iter_mx(SideLayout lay, SideVals<double> v64, SideVals<LowT<LP>> v32, WalkScratch wa,
-              WalkScratch wb, ColVecsMx v, const float *__restrict__ dyt,
-              const double *__restrict__ dyt64, const double *__restrict__ y0, Ctl *ctl,
-              double *part, IterConsts ic, int phase) {
+k_row_iter_mx(SideLayout lay, SideVals<double> v64, SideVals<LowT<LP>> v32, WalkScratch wa,
+              WalkScratch wb, RowVecsMx v, const float *__restrict__ dxt,
+              const double *__restrict__ dxt64, const double *__restrict__ x0, Ctl *ctl,
+              double *part, IterConsts ic, DeferredCol dc) {
   extern __shared__ double smem[];
-  if (ctl->status != kRunning || ctl->stage != 1) return;
+  if (ctl->status != kRunning) return;
+  if constexpr (MODE == 2) {
+    if (ctl->restart_pending)
+      row_iter_mx<RHO2, 1, kWalkGrouped, 0, LP, 0>(smem, lay, v64, v32, wa, wb, v, dxt, dxt64, x0,
+                                                   ctl, part, ic, dc);
+    else
+      row_iter_mx<RHO2, 0, WALK, DFS, LP, CP>(smem, lay, v64, v32, wa, wb, v, dxt, dxt64, x0, ctl,
+                                              part, ic, dc);
+  } else {
+    row_iter_mx<RHO2, MODE, WALK, DFS, LP, CP>(smem, lay, v64, v32, wa, wb, v, dxt, dxt64, x0, ctl,
+                                               part, ic, dc);
+  }
+}
+
+// MODE 0: ordinary iterations (no pending restart, not a restart point); MODE 1: the rest.
+template <int RHO2, int MODE, int WALK, int DFS, int LP, int CP>
+__device__ __forceinline__ void
+col_iter_mx(double *smem, const SideLayout &lay, const SideVals<double> v64,
+            const SideVals<LowT<LP>> v32, const WalkScratch wa, const WalkScratch wb,
+            const ColVecsMx &v, const float *__restrict__ dyt, const double *__restrict__ dyt64,
+            const double *__restrict__ y0, Ctl *ctl, double *part, const IterConsts &ic,
+            int phase) {
+  if (ctl->stage != 1) return;
   const long long t = ctl->t, k = ctl->k, n_ep = ctl->n;
   const int restart = ctl->restart_pending;
   const bool rp = phase == 0 && (k == 0 && n_ep >= 1);
@@ -247,6 +271,27 @@ k_col_iter_mx(SideLayout lay, SideVals<double> v64, SideVals<LowT<LP>> v32, Walk
   }
 }
 
+template <int RHO2, int MODE, int WALK, int DFS, int LP, int CP = 0>
+__global__ void __maxnreg__(mx_max_regs(MODE, WALK, DFS))
+k_col_iter_mx(SideLayout lay, SideVals<double> v64, SideVals<LowT<LP>> v32, WalkScratch wa,
+              WalkScratch wb, ColVecsMx v, const float *__restrict__ dyt,
+              const double *__restrict__ dyt64, const double *__restrict__ y0, Ctl *ctl,
+              double *part, IterConsts ic, int phase) {
+  extern __shared__ double smem[];
+  if (ctl->status != kRunning) return;
+  if constexpr (MODE == 2) {
+    if (ctl->restart_pending || (phase == 0 && ctl->k == 0 && ctl->n >= 1))
+      col_iter_mx<RHO2, 1, kWalkGrouped, 0, LP, 0>(smem, lay, v64, v32, wa, wb, v, dyt, dyt64, y0,
+                                                   ctl, part, ic, phase);
+    else
+      col_iter_mx<RHO2, 0, WALK, DFS, LP, CP>(smem, lay, v64, v32, wa, wb, v, dyt, dyt64, y0, ctl,
+                                              part, ic, phase);
+  } else {
+    col_iter_mx<RHO2, MODE, WALK, DFS, LP, CP>(smem, lay, v64, v32, wa, wb, v, dyt, dyt64, y0, ctl,
+                                               part, ic, phase);
+  }
+}
+
 // unscaled outputs: x = E (x0 + dxt) is already xout's E-image at checks; y = D (y0 + dyt)
 __global__ void k_unscale_mx(int n, int m, const double *e, const double *xs, const double *d,
                              const double *y0, const float *dyt, double *xo, double *yo,
@@ -268,7 +313,7 @@ __global__ void k_zero_f32(int n, float *x) {
 }  // namespace
 
 // The restart-mode kernel (MODE 1) of each stage is launched first and returns at entry unless
-// the stage needs it; the ordinary kernel (MODE 0) follows, in the instantiation of the side's
+// the stage needs it (both: one kernel, MODE 2, in their place); the ordinary kernel (MODE 0) follows, in the instantiation of the side's
 // walk (SideLayout::walk) and of the solve's restart-norm sums (IterConsts::df_sums).
 template <int V>
 using IC = std::integral_constant<int, V>;
@@ -294,13 +339,18 @@ void with_rho_dfs(int rho2, int dfs, F &&f) {
 void launch_row_iter_mx(cudaStream_t st, const SideStore &side, const RowVecsMx &v,
                         const float *dxt, const double *dxt64, const double *x0, Ctl *ctl,
                         double *part, const IterConsts &ic, int grid, int grid1, int smem,
-                        const DeferredCol &dc) {
+                        bool both, const DeferredCol &dc) {
   const int threads = side.lay.cta_warps * kWarp;
   auto go = [&](auto kern, int g, int sm, auto vals) {
     kern<<<g, threads, sm, st>>>(side.lay, side.v64, vals, side.wa, side.wb, v, dxt, dxt64, x0,
                                  ctl, part, ic, dc);
   };
   with_rho_dfs(ic.rho2, ic.df_sums, [&](auto R, auto D) {
+    if (both) {
+      with_walk<true>(side.lay.walk,
+                      [&](auto W) { go(k_row_iter_mx<R(), 2, W(), 0, 0>, grid, smem, side.v32); });
+      return;
+    }
     go(k_row_iter_mx<R(), 1, kWalkGrouped, 0, 0>, grid1, smem, side.v32);
     with_walk<true>(side.lay.walk, [&](auto W) {
       // evict-first matrix stream only for FP32 values with FP32 restart-norm sums (the
@@ -316,13 +366,18 @@ void launch_row_iter_mx(cudaStream_t st, const SideStore &side, const RowVecsMx 
 void launch_col_iter_mx(cudaStream_t st, const SideStore &side, const ColVecsMx &v,
                         const float *dyt, const double *dyt64, const double *y0, Ctl *ctl,
                         double *part, const IterConsts &ic, int grid, int grid1, int smem,
-                        int phase) {
+                        bool both, int phase) {
   const int threads = side.lay.cta_warps * kWarp;
   auto go = [&](auto kern, int g, int sm, auto vals) {
     kern<<<g, threads, sm, st>>>(side.lay, side.v64, vals, side.wa, side.wb, v, dyt, dyt64, y0,
                                  ctl, part, ic, phase);
   };
   with_rho_dfs(ic.rho2, ic.df_sums, [&](auto R, auto D) {
+    if (both) {
+      with_walk<false>(side.lay.walk,
+                       [&](auto W) { go(k_col_iter_mx<R(), 2, W(), 0, 0>, grid, smem, side.v32); });
+      return;
+    }
     go(k_col_iter_mx<R(), 1, kWalkGrouped, 0, 0>, grid1, smem, side.v32);
     with_walk<false>(side.lay.walk, [&](auto W) {
       const bool cp = ic.l2_first && ic.df_sums == 0;
@@ -356,11 +411,13 @@ void allow_large_smem_mx(int bytes) {
         set((const void *)k_col_iter_mx<R(), 1, kWalkGrouped, 0, 0>);
         for (int w : {kWalkPlain, kWalkWide, kWalkGrouped}) {
           with_walk<true>(w, [&](auto W) {
+            set((const void *)k_row_iter_mx<R(), 2, W(), 0, 0>);
             set((const void *)k_row_iter_mx<R(), 0, W(), D(), 0>);
             set((const void *)k_row_iter_mx<R(), 0, W(), 0, 1>);
             set((const void *)k_row_iter_mx<R(), 0, W(), 0, 0, 1>);
           });
           with_walk<false>(w, [&](auto W) {
+            set((const void *)k_col_iter_mx<R(), 2, W(), 0, 0>);
             set((const void *)k_col_iter_mx<R(), 0, W(), D(), 0>);
             set((const void *)k_col_iter_mx<R(), 0, W(), 0, 1>);
             set((const void *)k_col_iter_mx<R(), 0, W(), 0, 0, 1>);
@@ -383,6 +440,21 @@ int iter_mx_restart_blocks_per_sm(int smem, bool row, int threads) {
     occ((const void *)k_col_iter_mx<0, 1, kWalkGrouped, 0, 0>);
     occ((const void *)k_col_iter_mx<1, 1, kWalkGrouped, 0, 0>);
   }
+  return mn;
+}
+
+int iter_mx_both_blocks_per_sm(int smem, bool row, int walk, int threads) {
+  int mn = 1 << 30;
+  auto occ = [&](const void *f) {
+    int b = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, f, threads, smem);
+    mn = b < mn ? b : mn;
+  };
+  for (int rho2 = 0; rho2 < 2; ++rho2)
+    with_rho_dfs(rho2, 0, [&](auto R, auto) {
+      if (row) with_walk<true>(walk, [&](auto W) { occ((const void *)k_row_iter_mx<R(), 2, W(), 0, 0>); });
+      else with_walk<false>(walk, [&](auto W) { occ((const void *)k_col_iter_mx<R(), 2, W(), 0, 0>); });
+    });
   return mn;
 }
 

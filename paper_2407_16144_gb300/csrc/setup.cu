@@ -267,6 +267,7 @@ k_side_spmv_pw(SideLayout lay, SideVals<VT> vals, WalkScratch ws,
   auto gather = [&](int j) { return kF64 ? PT(src[j] * sc) : src[j]; };
   auto gdone = [&](int grp) { store_group(al, 0x1u, ws.group_part, grp); };
   walk_tiles<VT, PT>(lay, vals, gather, my, ws, epi, gdone);
+  if (!ss) return;       // a product whose norm nothing reads (every K^ v but the last)
   if (cta_reduce_and_ticket(a, 0x1u, 0u, 0u, part, ticket)) {
     double r[1];
     grid_finish<1, 0>(part, r, 0x1u, 0u, ws.group_part, lay.n_long_tiles);
