@@ -78,7 +78,7 @@ struct rhpdhg_handle {
   int col_rows_last = 1;              // CTA rows the last column launch wrote (see DeferredCol)
   double eta = 1.0, omega0 = 1.0, sigma_max = 0.0;
 
-  cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+  cudaGraphExec_t gexec = nullptr;     // one chunk of the stage kernels
   std::thread th;
   std::atomic<int> running{0};
   std::atomic<int> cancel{0};
@@ -128,12 +128,52 @@ cudaError_t dalloc(T **p, size_t count) {
   return buf_alloc((void **)p, (count > 0 ? count : 1) * sizeof(T));
 }
 
+// Pinned mirrors of freed handles, for later ones: pinning and unpinning a page takes 0.1 ms each.
+// At most kMirrors are held; rhpdhg_release_cached_memory gives them back.
+constexpr size_t kMirrors = 64;
+std::mutex g_mirror_mu;
+std::vector<Ctl *> g_mirrors;
+
+cudaError_t mirror_alloc(Ctl **p) {
+  {
+    std::lock_guard<std::mutex> lk(g_mirror_mu);
+    if (!g_mirrors.empty()) {
+      *p = g_mirrors.back();
+      g_mirrors.pop_back();
+      return cudaSuccess;
+    }
+  }
+  return cudaHostAlloc((void **)p, 2 * sizeof(Ctl), cudaHostAllocPortable);
+}
+
+void mirror_release(Ctl *p) {
+  if (!p) return;
+  {
+    std::lock_guard<std::mutex> lk(g_mirror_mu);
+    if (g_mirrors.size() < kMirrors) {
+      g_mirrors.push_back(p);
+      return;
+    }
+  }
+  cudaFreeHost(p);
+}
+
+void mirrors_drop() {
+  std::lock_guard<std::mutex> lk(g_mirror_mu);
+  for (Ctl *p : g_mirrors) cudaFreeHost(p);
+  g_mirrors.clear();
+}
+
+void drop_graph(rhpdhg_handle *h) {
+  if (h->gexec) cudaGraphExecDestroy(h->gexec);
+  h->gexec = nullptr;
+}
+
 void destroy(rhpdhg_handle *h) {
   if (!h) return;
   if (h->th.joinable()) h->th.join();
   if (h->st) cudaStreamSynchronize(h->st);
-  for (auto &g : h->gexec)
-    if (g) cudaGraphExecDestroy(g);
+  drop_graph(h);
   free_side(&h->rows);
   free_side(&h->cols);
   double *bufs[] = {h->D, h->E, h->Dinv, h->Einv, h->c, h->q, h->l, h->u, h->x, h->xt, h->x0,
@@ -147,7 +187,7 @@ void destroy(rhpdhg_handle *h) {
   buf_release(h->act);
   buf_release(h->ctl);
   buf_release(h->trace);
-  if (h->h_mirror) cudaFreeHost(h->h_mirror);
+  mirror_release(h->h_mirror);
   if (h->own_stream && h->st) cudaStreamDestroy(h->st);
   delete h;
 }
@@ -304,18 +344,18 @@ void launch_iteration(rhpdhg_handle *h) {
 constexpr int kMaxChunk = 256;
 int chunk_iters(const rhpdhg_handle *h) { return std::min(h->p.check_every, kMaxChunk); }
 
-int capture_graphs(rhpdhg_handle *h) {
-  for (int g = 0; g < 2; ++g) {
-    if (h->gexec[g]) continue;
-    cudaGraph_t graph;
-    CK(cudaStreamBeginCapture(h->st, cudaStreamCaptureModeThreadLocal));
-    for (int i = 0; i < chunk_iters(h); ++i) launch_iteration(h);
-    cudaMemcpyAsync(h->h_mirror + g, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, h->st);
-    CK(cudaStreamEndCapture(h->st, &graph));
-    cudaError_t e = cudaGraphInstantiate(&h->gexec[g], graph, 0);
-    cudaGraphDestroy(graph);
-    CK(e);
-  }
+// The chunk's launches as a graph; the copy of the control block follows each launch of it (two
+// graphs that differed in the mirror they ended with cost a second capture and instantiation per
+// handle, about 0.8 ms).
+int capture_graph(rhpdhg_handle *h) {
+  if (h->gexec) return RHPDHG_OK;
+  cudaGraph_t graph;
+  CK(cudaStreamBeginCapture(h->st, cudaStreamCaptureModeThreadLocal));
+  for (int i = 0; i < chunk_iters(h); ++i) launch_iteration(h);
+  CK(cudaStreamEndCapture(h->st, &graph));
+  const cudaError_t e = cudaGraphInstantiate(&h->gexec, graph, 0);
+  cudaGraphDestroy(graph);
+  CK(e);
   return RHPDHG_OK;
 }
 
@@ -364,8 +404,7 @@ int escalate_to_fp64(rhpdhg_handle *h) {
   CK(cudaMemcpy(&c, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
   h->mixed = false;
   h->ic.mixed = 0;
-  for (auto &g : h->gexec)
-    if (g) { cudaGraphExecDestroy(g); g = nullptr; }
+  drop_graph(h);
   CK(cudaMemcpyAsync(h->xt, h->x0, h->n * sizeof(double), cudaMemcpyDeviceToDevice, h->st));
   if (h->m)
     CK(cudaMemcpyAsync(h->yt, h->y0, h->m * sizeof(double), cudaMemcpyDeviceToDevice, h->st));
@@ -554,14 +593,13 @@ void drive(rhpdhg_handle *h) {
   if (h->created_mixed && !h->mixed) {      // a previous solve escalated: back to mixed
     h->mixed = true;
     h->ic.mixed = 1;
-    for (auto &g : h->gexec)
-      if (g) { cudaGraphExecDestroy(g); g = nullptr; }
+    drop_graph(h);
   }
   h->escalated = false;
   int rc = reset_state(h);
   h->launches += h->mixed ? 8 : 2;   // set-up kernels of the solve
   const bool graphs = h->p.use_graphs && !h->p.profile;
-  if (rc == RHPDHG_OK && graphs) rc = capture_graphs(h);
+  if (rc == RHPDHG_OK && graphs) rc = capture_graph(h);
   if (rc != RHPDHG_OK) {
     h->drive_err = rc;
     h->final_status = kNumericalError;
@@ -584,19 +622,22 @@ void drive(rhpdhg_handle *h) {
   // own pinned mirror; the host reads mirror g only after chunk g's event, and relaunches g
   // only after that read.
   const long long depth = h->p.profile ? 1 : 2;
-  long long last_t = 0;
+  long long last_t = 0, start_t = 0;
   int host_status = kRunning;
   for (;;) {
     long long launched = 0, done = 0;
+    const long long left = h->p.max_iters - start_t;   // iterations to the limit
     bool stop = false;
     int dev_status = kRunning;
     while (true) {
-      while (!stop && launched - done < depth) {
+      // (no further chunk behind one that reaches the iteration limit, unless that one left the
+      // solve running: rejected adaptive steps do not count)
+      while (!stop && launched - done < depth && (launched == done || launched * chunk < left)) {
         if (h->cancel.load()) { host_status = kCancelled; stop = true; break; }
         if (timer.s() > h->p.time_limit_s) { host_status = kTimeLimit; stop = true; break; }
         const int g = (int)(launched & 1);
         if (graphs) {
-          cudaGraphLaunch(h->gexec[g], h->st);
+          cudaGraphLaunch(h->gexec, h->st);
         } else {
           for (int i = 0; i < chunk; ++i) {
             if (h->p.profile) cudaEventRecord(pev[3 * i], h->st);
@@ -605,8 +646,8 @@ void drive(rhpdhg_handle *h) {
             launch_col(h, 0);
             if (h->p.profile) cudaEventRecord(pev[3 * i + 2], h->st);
           }
-          cudaMemcpyAsync(h->h_mirror + g, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, h->st);
         }
+        cudaMemcpyAsync(h->h_mirror + g, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, h->st);
         cudaEventRecord(ev[g], h->st);
         ++launched;
         h->launches += launches_per_iter(h) * chunk;
@@ -644,10 +685,10 @@ void drive(rhpdhg_handle *h) {
     }
     cudaStreamSynchronize(h->st);
     if (dev_status == kEscalate && host_status == kRunning && !h->drive_err) {
-      if (escalate_to_fp64(h) == RHPDHG_OK && (!graphs || capture_graphs(h) == RHPDHG_OK)) {
+      if (escalate_to_fp64(h) == RHPDHG_OK && (!graphs || capture_graph(h) == RHPDHG_OK)) {
         Ctl c{};
         cudaMemcpy(&c, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost);
-        last_t = c.t;
+        last_t = start_t = c.t;
         continue;
       }
       h->drive_err = RHPDHG_ERR_CUDA;
@@ -1035,7 +1076,7 @@ int rhpdhg_create(const rhpdhg_problem *lp, const rhpdhg_params *params, void *c
   if (m) CKC(cudaMemsetAsync(h->certy, 0, m * sizeof(double), st));
   if (m) CKC(cudaMemsetAsync(h->certy2, 0, m * sizeof(double), st));
   CKC(dalloc(&h->ctl, 1));
-  CKC(cudaHostAlloc((void **)&h->h_mirror, 2 * sizeof(Ctl), cudaHostAllocDefault));
+  CKC(mirror_alloc(&h->h_mirror));
   std::memset(h->h_mirror, 0, 2 * sizeof(Ctl));
   {
     int gr = h->grid_row, gc = h->grid_col;
@@ -1218,7 +1259,10 @@ int rhpdhg_get_layout(const rhpdhg_handle *h, int64_t *out, int32_t capacity) {
   return RHPDHG_OK;
 }
 
-int64_t rhpdhg_release_cached_memory(void) { return (int64_t)buf_drop_cache(); }
+int64_t rhpdhg_release_cached_memory(void) {
+  mirrors_drop();
+  return (int64_t)buf_drop_cache();
+}
 
 int rhpdhg_plan_layout(const int64_t *row_ptr, int32_t nrows, int64_t *out, int32_t capacity) {
   if (!row_ptr || !out || nrows < 0 || capacity < RHPDHG_PLAN_FIELDS || row_ptr[0] != 0)
