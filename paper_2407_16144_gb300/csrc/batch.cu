@@ -27,7 +27,13 @@ namespace rh {
 
 namespace {
 
-constexpr int kBT = 256;   // threads per CTA of the batched kernel
+// Threads per CTA of the batched kernel: 16 warps of at most 128 registers, a whole SM.  (8 warps of
+// 214 registers, also one CTA per SM, left half as many dependent loads in flight: 96 LPs of 100 to
+// 1600 rows, 256 iterations with set-up and transfers, 42.2 ms, now 31.5 with the passes' sums taken
+// together and the CTA's sums a slot per thread.)
+constexpr int kBT = 512;
+// Threads whose chains of FP32 restart-norm sums a slot's results are defined by (see replay_*).
+constexpr int kChain = 256;
 
 struct BatchDesc {
   int active;              // 1 = slot in use
@@ -64,43 +70,36 @@ __device__ __forceinline__ double group_max(double v, int g) {
 }
 
 // Block reduction of the NS sums and NM maxima selected by the masks into out (valid in thread
-// 0; other slots 0); deterministic.  Sum slots set in prewarp already hold their warp's sum.
+// 0; other slots 0); deterministic: warps in index order, a slot per thread of the first warp.  Sum
+// slots set in prewarp already hold their warp's sum, and only in the warps of the first kChain
+// threads.  sh: a row of kMaxPartials per warp, and one more.
 template <int NS, int NM>
-__device__ void block_reduce(const Acc<NS, NM> &a, double *out, double *sh,
+__device__ void block_reduce(Acc<NS, NM> &a, double *out, double (*sh)[kMaxPartials],
                              unsigned smask = 0xFFFFu, unsigned mmask = 0xFFFFu,
                              unsigned prewarp = 0u) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned all = (smask & ((1u << NS) - 1u)) | ((mmask & ((1u << NM) - 1u)) << NS);
+  const int tid = threadIdx.x;
+  smask &= (1u << NS) - 1u;
+  mmask &= (1u << NM) - 1u;
   __syncthreads();
-#pragma unroll
-  for (int i = 0; i < NS + NM; ++i) {
-    if (!((all >> i) & 1u)) continue;
-    double v = i < NS ? a.s[i] : a.mx[i - NS];
-    if (i >= NS) v = warp_max(v);
-    else if (!((prewarp >> i) & 1u)) v = warp_sum(v);
-    if (lane == 0) sh[warp * (NS + NM) + i] = v;
+  warp_reduce_to<NS, NM, 0, true>(a, smask, mmask, prewarp, sh[tid >> 5]);
+  __syncthreads();
+  if (tid < NS + NM) {
+    double v = 0.0;
+    if (((smask | (mmask << NS)) >> tid) & 1u)
+      v = cta_slot<NS, NM, 0, true>(sh, tid, ((prewarp >> tid) & 1u ? kChain : kBT) / 32);
+    sh[kBT / 32][tid] = v;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < NS + NM; ++i) {
-      if (!((all >> i) & 1u)) { out[i] = 0.0; continue; }
-      double v = sh[i];
-      for (int w = 1; w < kBT / 32; ++w)
-        v = i < NS ? v + sh[w * (NS + NM) + i] : fmax(v, sh[w * (NS + NM) + i]);
-      out[i] = v;
-    }
-  }
-  __syncthreads();
+  if (tid == 0)
+    for (int i = 0; i < NS + NM; ++i) out[i] = sh[kBT / 32][i];
 }
 
-__device__ double block_sum1(double v, double *sh) {
+__device__ double block_sum1(double v, double (*sh)[kMaxPartials]) {
   Acc<1, 0> a;
   a.s[0] = v;
   double out[1] = {0.0};
   block_reduce(a, out, sh);
-  if (threadIdx.x == 0) sh[0] = out[0];
-  __syncthreads();
-  const double r = sh[0];
+  const double r = sh[kBT / 32][0];
   __syncthreads();
   return r;
 }
@@ -161,10 +160,26 @@ __device__ __forceinline__ void rows_apply(int nrows, const int *ptr, const int 
           if (p0[u] + t * g < pe[u]) s[u] += v[u][t] * x[u][t];
         for (int p = p0[u] + kRowSteps * g; p < pe[u]; p += g) s[u] += val[p] * VT(src(idx[p]));
       }
+      const int mypass = lane / rpp - pass0;        // the pass that sums this lane's own row
+      if (g >= 4) {
+        // all four passes' group sums at once: a lane keeps two of them, then one, and hands the
+        // others to its partner (the additions are those of group_sum, 4 + log2(g) - 3 instead of
+        // 4 log2(g) per lane)
+        static_assert(kRowPasses == 4, "two halvings");
+        const bool h2 = lane & (g / 2), h1 = lane & (g / 4);
+        const VT a0 = (h2 ? s[2] : s[0]) + __shfl_xor_sync(full, h2 ? s[0] : s[2], g / 2);
+        const VT a1 = (h2 ? s[3] : s[1]) + __shfl_xor_sync(full, h2 ? s[1] : s[3], g / 2);
+        VT r = (h1 ? a1 : a0) + __shfl_xor_sync(full, h1 ? a0 : a1, g / 4);
+        for (int o = g / 8; o > 0; o /= 2) r += __shfl_xor_sync(full, r, o);
+        const VT got = __shfl_sync(full, r, (lane % rpp) * g + (mypass >> 1 & 1) * (g / 2) +
+                                                (mypass & 1) * (g / 4));
+        if (mypass >= 0 && mypass < kRowPasses) mine = got;
+      } else {
 #pragma unroll
-      for (int u = 0; u < kRowPasses; ++u) {
-        const VT got = __shfl_sync(full, group_sum(s[u], g), (lane % rpp) * g);
-        if (lane / rpp == pass0 + u) mine = got;
+        for (int u = 0; u < kRowPasses; ++u) {
+          const VT got = __shfl_sync(full, group_sum(s[u], g), (lane % rpp) * g);
+          if (mypass == u) mine = got;
+        }
       }
     }
     if (row < nrows) fn(row, mine);
@@ -200,7 +215,7 @@ __device__ void scale_update(int n, const double *stat, double *scale) {
 }
 
 // The whole create-time pipeline of one LP, inside its CTA.
-__device__ void batch_setup(const BatchDesc &d, double *sh) {
+__device__ void batch_setup(const BatchDesc &d, double (*sh)[kMaxPartials]) {
   const int m = d.m, n = d.n;
   RowVecs rvv = d.rv_;
   ColVecs cvv = d.cv_;
@@ -282,8 +297,8 @@ __device__ void batch_setup(const BatchDesc &d, double *sh) {
       __syncthreads();
       double ss = 0.0;
       for (int j = threadIdx.x; j < n; j += kBT) ss += w[j] * w[j];
-      const double nrm = sqrt(block_sum1(ss, sh));
-      for (int j = threadIdx.x; j < n; j += kBT) v[j] = nrm > 0.0 ? w[j] / nrm : 0.0;
+      const double nrm = sqrt(block_sum1(ss, sh)), inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
+      for (int j = threadIdx.x; j < n; j += kBT) v[j] = w[j] * inv;
       __syncthreads();
     }
     auto f1 = [&](int r, double s) { um[r] = s; };
@@ -349,7 +364,7 @@ __device__ void batch_setup(const BatchDesc &d, double *sh) {
 }
 
 template <int RHO2>
-__device__ void batch_col_pass(const BatchDesc &d, const IterConsts &ic, int phase, double *sh) {
+__device__ void batch_col_pass(const BatchDesc &d, const IterConsts &ic, int phase, double (*sh)[kMaxPartials]) {
   Ctl *ctl = d.ctl;
   const long long t = ctl->t, k = ctl->k, n_ep = ctl->n;
   const bool check = phase == 0 && (((t + 1) % ic.check_every == 0) || (t + 1 >= ic.max_iters));
@@ -375,7 +390,7 @@ __device__ void batch_col_pass(const BatchDesc &d, const IterConsts &ic, int pha
 }
 
 template <int RHO2>
-__device__ void batch_row_pass(const BatchDesc &d, const IterConsts &ic, double *sh) {
+__device__ void batch_row_pass(const BatchDesc &d, const IterConsts &ic, double (*sh)[kMaxPartials]) {
   Ctl *ctl = d.ctl;
   const long long t = ctl->t, k = ctl->k, n_ep = ctl->n;
   const bool check = ((t + 1) % ic.check_every == 0) || (t + 1 >= ic.max_iters);
@@ -397,13 +412,59 @@ __device__ void batch_row_pass(const BatchDesc &d, const IterConsts &ic, double 
   __syncthreads();
 }
 
-// The FP32 restart-norm sums of a thread, summed over its warp in FP32 and placed in the FP64
-// slots of a (lane 0 holds the warp's sum; block_reduce adds the warps in FP64).
-template <int N, class A>
-__device__ __forceinline__ unsigned warp_sums_to(FprSums<N, 0> &f, A &a) {
-#pragma unroll
-  for (int i = 0; i < N; ++i) a.s[i] = (double)warp_sum(f.v[i].hi);
-  return (1u << N) - 1u;
+// The FP32 restart-norm sums of the ordinary iterations.  Their order decides their rounding, and
+// through the restart rule and the primal weight a slot's results, so it does not follow the CTA's
+// width: thread i of the first kChain adds rows i, i + kChain, ... in order, then each warp its lanes
+// in FP32 and the block its warps in FP64.  The pass over the rows leaves the factors (in the
+// set-up's scratch); these kernels add them up.
+struct RowFactors {          // of a row: y - y~ and K x - K x~ (y~ - y0 is kept in dyt)
+  float2 *at;
+  __device__ __forceinline__ void add(int i, float a, float b) {
+    if (i == 0) at->x = a;
+    if (i == 1) at->y = b;
+  }
+};
+struct ColFactors {          // of a column: x - x~ (x~ - x0 is kept in dxt)
+  float *at;
+  __device__ __forceinline__ void add(int i, float a, float) {
+    if (i == 0) *at = a;
+  }
+};
+// Both return the mask of the slots that hold their warp's sum.
+__device__ __forceinline__ unsigned replay_rows(int m, const float2 *f, const float *dyt,
+                                                Acc<7, 6> &a) {
+  __syncthreads();
+  float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+  if (threadIdx.x < kChain) {
+#pragma unroll 4
+    for (int i = threadIdx.x; i < m; i += kChain) {
+      const float2 p = f[i];
+      const float d = dyt[i];
+      s0 = __fmaf_rn(p.x, p.x, s0);
+      s1 = __fmaf_rn(p.x, p.y, s1);
+      s2 = __fmaf_rn(d, d, s2);
+    }
+    a.s[0] = (double)warp_sum(s0);
+    a.s[1] = (double)warp_sum(s1);
+    a.s[2] = (double)warp_sum(s2);
+  }
+  return 0x7u;
+}
+__device__ __forceinline__ unsigned replay_cols(int n, const float *f, const float *dxt,
+                                                Acc<11, 8> &a) {
+  __syncthreads();
+  float s0 = 0.f, s1 = 0.f;
+  if (threadIdx.x < kChain) {
+#pragma unroll 4
+    for (int j = threadIdx.x; j < n; j += kChain) {
+      const float d = f[j], e = dxt[j];
+      s0 = __fmaf_rn(d, d, s0);
+      s1 = __fmaf_rn(e, e, s1);
+    }
+    a.s[0] = (double)warp_sum(s0);
+    a.s[1] = (double)warp_sum(s1);
+  }
+  return 0x3u;
 }
 
 // ---- mixed precision in a slot: the bodies of the tiled mixed kernels (iter_mx_common.cuh) over
@@ -411,7 +472,7 @@ __device__ __forceinline__ unsigned warp_sums_to(FprSums<N, 0> &f, A &a) {
 // restart points; the restart-norm sums are FP32 within each warp and FP64 across the warps.
 
 template <int RHO2>
-__device__ void batch_row_pass_mx(const BatchDesc &d, const IterConsts &ic, double *sh) {
+__device__ void batch_row_pass_mx(const BatchDesc &d, const IterConsts &ic, double (*sh)[kMaxPartials]) {
   Ctl *ctl = d.ctl;
   const long long t = ctl->t, k = ctl->k, n_ep = ctl->n;
   const bool check = ((t + 1) % ic.check_every == 0) || (t + 1 >= ic.max_iters);
@@ -443,12 +504,15 @@ __device__ void batch_row_pass_mx(const BatchDesc &d, const IterConsts &ic, doub
     };
     rows_apply(d.m, d.rp, d.ci, d.rv, d.gr, gB, fB);
   } else {
-    FprSums<3, 0> f;
+    float2 *factors = reinterpret_cast<float2 *>(d.tmp_m);
     const float *dxt = d.cvm.dxt;
     auto g = [&](int j) { return dxt[j]; };
-    auto fn = [&](int i, float kd) { row_mx_ordinary<RHO2>(i, kd, v, wf, sigf, m_eq, check, a, f); };
+    auto fn = [&](int i, float kd) {
+      RowFactors f{factors + i};
+      row_mx_ordinary<RHO2>(i, kd, v, wf, sigf, m_eq, check, a, f);
+    };
     rows_apply(d.m, d.rp, d.ci, d.rv32, d.gr, g, fn);
-    prewarp = warp_sums_to(f, a);
+    prewarp = replay_rows(d.m, factors, v.dyt, a);
   }
   double r[13];
   block_reduce(a, r, sh, row_smask(check, rp, move), row_mmask(rp, move), prewarp);
@@ -458,7 +522,7 @@ __device__ void batch_row_pass_mx(const BatchDesc &d, const IterConsts &ic, doub
 
 template <int RHO2>
 __device__ void batch_col_pass_mx(const BatchDesc &d, const IterConsts &ic, int phase,
-                                  double *sh) {
+                                  double (*sh)[kMaxPartials]) {
   Ctl *ctl = d.ctl;
   const long long t = ctl->t, k = ctl->k, n_ep = ctl->n;
   const int restart = ctl->restart_pending;
@@ -489,15 +553,16 @@ __device__ void batch_col_pass_mx(const BatchDesc &d, const IterConsts &ic, int 
     };
     rows_apply(d.n, d.cp, d.ri, d.cv, d.gc, g, fn);
   } else {
-    FprSums<2, 0> f;
+    float *factors = reinterpret_cast<float *>(d.tmp_n);
     const float *dyt = d.rvm.dyt;
     auto g = [&](int i) { return dyt[i]; };
     auto fn = [&](int j, float ktdyt) {
+      ColFactors f{factors + j};
       col_mx_ordinary<RHO2>(j, ktdyt, v, wf, tauf, check, ic.no_upper, a, a, f, tl);
     };
     rows_apply(d.n, d.cp, d.ri, d.cv32, d.gc, g, fn);
     if (check) tel_flush(ctl, tl);
-    prewarp = warp_sums_to(f, a);
+    prewarp = replay_cols(d.n, factors, v.dxt, a);
   }
   double r[19];
   block_reduce(a, r, sh, col_smask(check, rp, move), col_mmask(rp, move), prewarp);
@@ -511,7 +576,7 @@ __device__ void batch_col_pass_mx(const BatchDesc &d, const IterConsts &ic, int 
 // starts there as at the start of a solve, with the iteration and epoch counters, the primal
 // weight and the step carried on, and the slot stays FP64.
 template <int RHO2>
-__device__ void batch_escalate(const BatchDesc &d, IterConsts &ic, double *sh) {
+__device__ void batch_escalate(const BatchDesc &d, IterConsts &ic, double (*sh)[kMaxPartials]) {
   const RowVecs &rv = d.rv_;
   const ColVecs &cv = d.cv_;
   for (int j = threadIdx.x; j < d.n; j += kBT) cv.xt[j] = cv.x0[j];
@@ -539,7 +604,7 @@ __device__ void batch_escalate(const BatchDesc &d, IterConsts &ic, double *sh) {
 }
 
 template <int RHO2>
-__device__ void batch_iterate(const BatchDesc &d, IterConsts &ic, int iters, double *sh) {
+__device__ void batch_iterate(const BatchDesc &d, IterConsts &ic, int iters, double (*sh)[kMaxPartials]) {
   Ctl *ctl = d.ctl;
   for (int it = 0; it < iters; ++it) {
     if (ctl->status == kEscalate) batch_escalate<RHO2>(d, ic, sh);
@@ -555,7 +620,7 @@ __device__ void batch_iterate(const BatchDesc &d, IterConsts &ic, int iters, dou
 
 __global__ void __launch_bounds__(kBT, 1)
 k_batch(const BatchDesc *__restrict__ descs, int nslots, int iters) {
-  __shared__ double sh[(kBT / 32) * kMaxPartials];
+  __shared__ double sh[kBT / 32 + 1][kMaxPartials];
   __shared__ IterConsts ics;
   // the slot's descriptor (registers are for the rows in flight) and its control block during the
   // launch (the finalisers are one thread's chains of reads and writes of it)
