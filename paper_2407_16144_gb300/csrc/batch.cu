@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "../../include/rhpdhg.h"
+#include "bufcache.h"
 #include "internal.h"
 #include "iter_common.cuh"
 #include "iter_mx_common.cuh"
@@ -659,16 +660,25 @@ k_batch(const BatchDesc *__restrict__ descs, int nslots, int iters) {
   if (threadIdx.x == 0) *home = ctls;
 }
 
-// Unscaled result of a slot: x = E x~ of the last check; y = D y~, where a slot still in mixed
-// precision holds y~ as y0 + dyt.
-__global__ void k_batch_unscale(const BatchDesc *__restrict__ descs, int slot, double *xo,
-                                double *yo) {
-  const BatchDesc d = descs[slot];
+// What a poll gives back of a slot, in one array: x = E x~ of the last check (n), y = D y~ (m),
+// where a slot still in mixed precision holds y~ as y0 + dyt, the certificate's parts (n, m) and
+// sigma_max.
+__global__ void k_batch_result(const BatchDesc *__restrict__ descs, int slot, int moved,
+                               double *out) {
+  const BatchDesc &d = descs[slot];
   const bool mixed = d.mixed && d.ic->mixed;
-  for (int j = threadIdx.x + blockIdx.x * blockDim.x; j < d.n; j += blockDim.x * gridDim.x)
-    xo[j] = d.cv_.e[j] * d.cv_.xout[j];
-  for (int i = threadIdx.x + blockIdx.x * blockDim.x; i < d.m; i += blockDim.x * gridDim.x)
+  const double *cx = moved ? d.cv_.certx2 : d.cv_.certx, *cy = moved ? d.rv_.certy2 : d.rv_.certy;
+  double *yo = out + d.n, *cxo = yo + d.m, *cyo = cxo + d.n;
+  const int at = threadIdx.x + blockIdx.x * blockDim.x, step = blockDim.x * gridDim.x;
+  for (int j = at; j < d.n; j += step) {
+    out[j] = d.cv_.e[j] * d.cv_.xout[j];
+    cxo[j] = cx[j];
+  }
+  for (int i = at; i < d.m; i += step) {
     yo[i] = d.rv_.d[i] * (mixed ? d.rvm.y0[i] + (double)d.rvm.dyt[i] : d.rv_.yt[i]);
+    cyo[i] = cy[i];
+  }
+  if (at == 0) cyo[d.m] = d.setup_out[0];
 }
 
 int pick_group(double avg) {
@@ -703,6 +713,12 @@ struct rhpdhg_batch {
   rh::BatchDesc *d_desc = nullptr;
   rh::Ctl *d_ctls = nullptr;               // every slot's control block (contiguous)
   rh::Ctl *h_ctl = nullptr;                // pinned copies of them
+  // pinned staging of an added LP's arrays (one copy to the arena instead of nine from pageable
+  // memory), free again when `staged` has passed; device and pinned copies of a polled result
+  char *h_stage = nullptr, *h_out = nullptr;
+  double *d_out = nullptr;
+  size_t stage_bytes = 0, out_bytes = 0;
+  cudaEvent_t staged = nullptr;
   cudaGraphExec_t gexec = nullptr;
   int graph_iters = -1;
   std::string err;
@@ -760,6 +776,35 @@ void arena_release(rhpdhg_batch *b, size_t off, size_t size) {
   }
 }
 
+// Grows the pinned staging area to at least `bytes`, once nothing in flight reads it.
+cudaError_t stage_reserve(rhpdhg_batch *b, size_t bytes) {
+  cudaError_t e = cudaEventSynchronize(b->staged);
+  if (e != cudaSuccess || bytes <= b->stage_bytes) return e;
+  cudaFreeHost(b->h_stage);
+  b->h_stage = nullptr;
+  b->stage_bytes = 0;
+  bytes += bytes / 2;
+  e = cudaHostAlloc((void **)&b->h_stage, bytes, cudaHostAllocDefault);
+  if (e == cudaSuccess) b->stage_bytes = bytes;
+  return e;
+}
+
+// Grows the two copies of a polled result (the stream is idle: every poll ends with a
+// synchronisation).
+cudaError_t out_reserve(rhpdhg_batch *b, size_t bytes) {
+  if (bytes <= b->out_bytes) return cudaSuccess;
+  rh::buf_release(b->d_out);
+  cudaFreeHost(b->h_out);
+  b->d_out = nullptr;
+  b->h_out = nullptr;
+  b->out_bytes = 0;
+  bytes += bytes / 2;
+  cudaError_t e = rh::buf_alloc((void **)&b->d_out, bytes);
+  if (e == cudaSuccess) e = cudaHostAlloc((void **)&b->h_out, bytes, cudaHostAllocDefault);
+  if (e == cudaSuccess) b->out_bytes = bytes;
+  return e;
+}
+
 int berr(rhpdhg_batch *b, int code, const std::string &msg) {
   if (b) b->err = msg;
   rh::set_global_error(msg);
@@ -789,6 +834,7 @@ int rhpdhg_batch_create(int32_t max_slots, int64_t arena_bytes, void *cuda_strea
   if (e == cudaSuccess) e = cudaMalloc(&b->d_desc, max_slots * sizeof(rh::BatchDesc));
   if (e == cudaSuccess) e = cudaMalloc(&b->d_ctls, max_slots * sizeof(rh::Ctl));
   if (e == cudaSuccess) e = cudaHostAlloc((void **)&b->h_ctl, max_slots * sizeof(rh::Ctl), 0);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->staged, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     rhpdhg_batch_free(b);
     return berr(nullptr, RHPDHG_ERR_OOM, std::string("batch: ") + cudaGetErrorString(e));
@@ -835,11 +881,9 @@ int rhpdhg_batch_add(rhpdhg_batch *b, const rhpdhg_problem *lp, const rhpdhg_par
   // host validation and transpose (the batched path serves small LPs)
   const int64_t *rp = lp->row_ptr;
   if (rp[0] != 0 || rp[m] != nnz) return berr(b, RHPDHG_ERR_INVALID_ARG, "batch: malformed row_ptr");
-  std::vector<int> rp32(m + 1), ci(nnz), cp(n + 2, 0), ri(nnz);
-  std::vector<double> cv(nnz);
+  std::vector<int> cp(n + 2, 0);
   for (int i = 0; i < m; ++i) {
     if (rp[i + 1] < rp[i]) return berr(b, RHPDHG_ERR_INVALID_ARG, "batch: malformed row_ptr");
-    rp32[i] = (int)rp[i];
     int prev = -1;
     for (long long q = rp[i]; q < rp[i + 1]; ++q) {
       const int j = lp->col_idx[q];
@@ -847,12 +891,10 @@ int rhpdhg_batch_add(rhpdhg_batch *b, const rhpdhg_problem *lp, const rhpdhg_par
         return berr(b, RHPDHG_ERR_INVALID_ARG,
                     "batch: column index out of range / not increasing, or non-finite value");
       prev = j;
-      ci[q] = j;
       cp[j + 2]++;
     }
     if (!std::isfinite(lp->rhs[i])) return berr(b, RHPDHG_ERR_INVALID_ARG, "batch: non-finite rhs");
   }
-  rp32[m] = (int)nnz;
   bool any_upper = false;
   for (int j = 0; j < n; ++j) {
     if (!std::isfinite(lp->c[j]) || std::isnan(lp->l[j]) || std::isnan(lp->u[j]) ||
@@ -861,14 +903,6 @@ int rhpdhg_batch_add(rhpdhg_batch *b, const rhpdhg_problem *lp, const rhpdhg_par
     any_upper = any_upper || std::isfinite(lp->u[j]);
   }
   for (int j = 0; j < n; ++j) cp[j + 2] += cp[j + 1];
-  for (int i = 0; i < m; ++i)
-    for (long long q = rp[i]; q < rp[i + 1]; ++q) {
-      const int j = ci[q];
-      const int pos = cp[j + 1]++;
-      ri[pos] = i;
-      cv[pos] = lp->val[q];
-    }
-  cp.resize(n + 1);
   // slot and arena region
   int slot = -1;
   for (int s = 0; s < b->max_slots; ++s)
@@ -896,26 +930,30 @@ int rhpdhg_batch_add(rhpdhg_batch *b, const rhpdhg_problem *lp, const rhpdhg_par
   d.step_size = P.step_size;
   d.step_safety = P.step_safety;
   d.primal_weight = P.primal_weight;
+  // the arrays copied from the host first, one after the other, then those that start at zero
+  const size_t nb = (size_t)std::max(n, 1) * 8, mb = (size_t)std::max(m, 1) * 8;
   int *d_rp = (int *)take((m + 1) * sizeof(int));
   int *d_ci = (int *)take(nnz * sizeof(int));
   double *d_rv = (double *)take(nnz * 8);
   int *d_cp = (int *)take((n + 1) * sizeof(int));
   int *d_ri = (int *)take(nnz * sizeof(int));
   double *d_cv = (double *)take(nnz * 8);
+  double *c = (double *)take(nb), *l = (double *)take(nb), *u = (double *)take(nb),
+         *q = (double *)take(mb);
+  rh::IterConsts *ic = (rh::IterConsts *)take(sizeof(rh::IterConsts));
+  const size_t upload = cur;
+  double *certx = (double *)take(nb), *certx2 = (double *)take(nb), *certy = (double *)take(mb),
+         *certy2 = (double *)take(mb);
+  unsigned char *act = (unsigned char *)take((size_t)std::max(n, 1));
+  const size_t zeroed = cur - upload;
   d.rp = d_rp; d.ci = d_ci; d.rv = d_rv; d.cp = d_cp; d.ri = d_ri; d.cv = d_cv;
-  const size_t nb = (size_t)std::max(n, 1) * 8, mb = (size_t)std::max(m, 1) * 8;
   double *x = (double *)take(nb), *xt = (double *)take(nb), *x0 = (double *)take(nb),
          *kty = (double *)take(nb), *kty0 = (double *)take(nb), *xout = (double *)take(nb),
-         *certx = (double *)take(nb), *c = (double *)take(nb), *l = (double *)take(nb),
-         *u = (double *)take(nb), *E = (double *)take(nb), *Einv = (double *)take(nb),
-         *tmp_n = (double *)take(nb), *certx2 = (double *)take(nb);
-  unsigned char *act = (unsigned char *)take((size_t)std::max(n, 1));
+         *E = (double *)take(nb), *Einv = (double *)take(nb), *tmp_n = (double *)take(nb);
   double *y = (double *)take(mb), *yt = (double *)take(mb), *y0 = (double *)take(mb),
          *kx = (double *)take(mb), *kxt = (double *)take(mb), *kx0 = (double *)take(mb),
-         *certy = (double *)take(mb), *q = (double *)take(mb), *D = (double *)take(mb),
-         *Dinv = (double *)take(mb), *tmp_m = (double *)take(mb), *certy2 = (double *)take(mb);
+         *D = (double *)take(mb), *Dinv = (double *)take(mb), *tmp_m = (double *)take(mb);
   rh::Ctl *ctl = b->d_ctls + slot;
-  rh::IterConsts *ic = (rh::IterConsts *)take(sizeof(rh::IterConsts));
   double *setup_out = (double *)take(16);
   d.tmp_m = tmp_m;
   d.tmp_n = tmp_n;
@@ -939,24 +977,6 @@ int rhpdhg_batch_add(rhpdhg_batch *b, const rhpdhg_problem *lp, const rhpdhg_par
   d.ctl = ctl;
   d.ic = ic;
   d.setup_out = setup_out;
-  cudaStream_t st = b->st;
-  cudaMemcpyAsync(d_rp, rp32.data(), (m + 1) * sizeof(int), cudaMemcpyHostToDevice, st);
-  if (nnz) {
-    cudaMemcpyAsync(d_ci, ci.data(), nnz * sizeof(int), cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(d_rv, lp->val, nnz * 8, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(d_ri, ri.data(), nnz * sizeof(int), cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(d_cv, cv.data(), nnz * 8, cudaMemcpyHostToDevice, st);
-  }
-  cudaMemcpyAsync(d_cp, cp.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(c, lp->c, n * 8, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(l, lp->l, n * 8, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(u, lp->u, n * 8, cudaMemcpyHostToDevice, st);
-  if (m) cudaMemcpyAsync(q, lp->rhs, m * 8, cudaMemcpyHostToDevice, st);
-  cudaMemsetAsync(certx, 0, nb, st);
-  cudaMemsetAsync(certy, 0, mb, st);
-  cudaMemsetAsync(certx2, 0, nb, st);
-  cudaMemsetAsync(act, 0, (size_t)std::max(n, 1), st);
-  cudaMemsetAsync(certy2, 0, mb, st);
   rh::Ctl c0{};
   c0.status = rh::kRunning;
   c0.stage = 2;                     // set-up pending
@@ -978,12 +998,48 @@ int rhpdhg_batch_add(rhpdhg_batch *b, const rhpdhg_problem *lp, const rhpdhg_par
   ic0.trace = nullptr;
   ic0.mixed = mixed ? 1 : 0;
   ic0.no_upper = any_upper ? 0 : 1;
-  // the host copies must outlive the async copies: stage through a synchronisation
-  cudaMemcpyAsync(ctl, &c0, sizeof(c0), cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(ic, &ic0, sizeof(ic0), cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(b->d_desc + slot, &d, sizeof(d), cudaMemcpyHostToDevice, st);
-  cudaError_t e = cudaStreamSynchronize(st);
+  // staged in pinned memory at the arena's offsets, the control block and descriptor behind them
+  cudaStream_t st = b->st;
+  const size_t at_ctl = upload, at_desc = at_ctl + align256(sizeof(c0));
+  cudaError_t e = stage_reserve(b, at_desc + align256(sizeof(d)));
   if (e != cudaSuccess) {
+    cudaGetLastError();
+    arena_release(b, off, need);
+    return berr(b, e == cudaErrorMemoryAllocation ? RHPDHG_ERR_OOM : RHPDHG_ERR_CUDA,
+                std::string("batch add: ") + cudaGetErrorString(e));
+  }
+  auto host = [&](const void *dev) { return b->h_stage + ((const char *)dev - base); };
+  int *rp32 = (int *)host(d_rp), *h_cp = (int *)host(d_cp), *h_ri = (int *)host(d_ri);
+  double *h_cv = (double *)host(d_cv);
+  for (int i = 0; i <= m; ++i) rp32[i] = (int)rp[i];
+  for (int i = 0; i < m; ++i)
+    for (long long t = rp[i]; t < rp[i + 1]; ++t) {
+      const int pos = cp[lp->col_idx[t] + 1]++;
+      h_ri[pos] = i;
+      h_cv[pos] = lp->val[t];
+    }
+  std::memcpy(h_cp, cp.data(), (n + 1) * sizeof(int));
+  if (nnz) {
+    std::memcpy(host(d_ci), lp->col_idx, nnz * sizeof(int));
+    std::memcpy(host(d_rv), lp->val, nnz * 8);
+  }
+  std::memcpy(host(c), lp->c, n * 8);
+  std::memcpy(host(l), lp->l, n * 8);
+  std::memcpy(host(u), lp->u, n * 8);
+  if (m) std::memcpy(host(q), lp->rhs, m * 8);
+  std::memcpy(host(ic), &ic0, sizeof(ic0));
+  std::memcpy(b->h_stage + at_ctl, &c0, sizeof(c0));
+  std::memcpy(b->h_stage + at_desc, &d, sizeof(d));
+  e = cudaMemcpyAsync(base, b->h_stage, upload, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(certx, 0, zeroed, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(ctl, b->h_stage + at_ctl, sizeof(c0), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(b->d_desc + slot, b->h_stage + at_desc, sizeof(d), cudaMemcpyHostToDevice,
+                        st);
+  if (e == cudaSuccess) e = cudaEventRecord(b->staged, st);
+  if (e != cudaSuccess) {
+    cudaStreamSynchronize(st);
     arena_release(b, off, need);
     return berr(b, RHPDHG_ERR_CUDA, std::string("batch add: ") + cudaGetErrorString(e));
   }
@@ -1042,28 +1098,39 @@ int rhpdhg_batch_poll(rhpdhg_batch *b, int32_t slot, rhpdhg_result *r) {
   r->solve_seconds = 0.0;
   r->eta = c.eta;
   r->omega = c.omega;
-  double so[2] = {0, 0};
-  cudaMemcpyAsync(so, d.setup_out, 16, cudaMemcpyDeviceToHost, b->st);
   const int m = d.m, n = d.n;
-  double *xo = nullptr, *yo = nullptr;
-  cudaMalloc(&xo, (size_t)std::max(n, 1) * 8);
-  cudaMalloc(&yo, (size_t)std::max(m, 1) * 8);
-  rh::k_batch_unscale<<<4, 256, 0, b->st>>>(b->d_desc, slot, xo, yo);
-  b->launches += 1;
-  const cudaMemcpyKind kind =
-      r->out_memory == RHPDHG_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  if (r->x) cudaMemcpyAsync(r->x, xo, n * 8, kind, b->st);
-  if (r->y && m) cudaMemcpyAsync(r->y, yo, m * 8, kind, b->st);
   const bool mv = c.cert_src == rh::kCertAnchorMove;
   r->cert_source = c.cert_src;
-  if (r->cert_x) cudaMemcpyAsync(r->cert_x, mv ? d.cv_.certx2 : d.cv_.certx, n * 8, kind, b->st);
-  if (r->cert_y && m)
-    cudaMemcpyAsync(r->cert_y, mv ? d.rv_.certy2 : d.rv_.certy, m * 8, kind, b->st);
-  cudaError_t e = cudaStreamSynchronize(b->st);
-  cudaFree(xo);
-  cudaFree(yo);
-  r->sigma_max = so[0];
+  const size_t count = 2 * ((size_t)n + m) + 1;
+  cudaError_t e = out_reserve(b, count * sizeof(double));
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return berr(b, e == cudaErrorMemoryAllocation ? RHPDHG_ERR_OOM : RHPDHG_ERR_CUDA,
+                std::string("batch poll: ") + cudaGetErrorString(e));
+  }
+  const int blocks = std::min(64, (std::max(n, m) + 255) / 256);
+  rh::k_batch_result<<<blocks, 256, 0, b->st>>>(b->d_desc, slot, mv ? 1 : 0, b->d_out);
+  b->launches += 1;
+  // the four vectors' places in the result and in the caller's buffers
+  const struct { double *to; size_t at, len; } parts[4] = {
+      {r->x, 0, (size_t)n}, {r->y, (size_t)n, (size_t)m},
+      {r->cert_x, (size_t)n + m, (size_t)n}, {r->cert_y, 2 * (size_t)n + m, (size_t)m}};
+  const bool device = r->out_memory == RHPDHG_MEM_DEVICE;
+  if (device) {
+    for (const auto &p : parts)
+      if (p.to && p.len)
+        cudaMemcpyAsync(p.to, b->d_out + p.at, p.len * 8, cudaMemcpyDeviceToDevice, b->st);
+    cudaMemcpyAsync(b->h_out, b->d_out + count - 1, 8, cudaMemcpyDeviceToHost, b->st);
+  } else {
+    cudaMemcpyAsync(b->h_out, b->d_out, count * 8, cudaMemcpyDeviceToHost, b->st);
+  }
+  e = cudaStreamSynchronize(b->st);
   if (e != cudaSuccess) return berr(b, RHPDHG_ERR_CUDA, cudaGetErrorString(e));
+  const double *got = (const double *)b->h_out;
+  r->sigma_max = device ? got[0] : got[count - 1];
+  if (!device)
+    for (const auto &p : parts)
+      if (p.to && p.len) std::memcpy(p.to, got + p.at, p.len * 8);
   return RHPDHG_OK;
 }
 
@@ -1072,9 +1139,8 @@ int rhpdhg_batch_remove(rhpdhg_batch *b, int32_t slot) {
     return RHPDHG_ERR_INVALID_ARG;
   rh::BatchDesc d{};
   d.active = 0;
-  cudaMemcpyAsync(b->d_desc + slot, &d, sizeof(d), cudaMemcpyHostToDevice, b->st);
+  cudaMemsetAsync(b->d_desc + slot, 0, sizeof(rh::BatchDesc), b->st);
   cudaMemsetAsync(b->d_ctls + slot, 0, sizeof(rh::Ctl), b->st);
-  cudaStreamSynchronize(b->st);
   arena_release(b, b->slot_region[slot].off, b->slot_region[slot].size);
   b->host_desc[slot] = d;
   b->slot_region[slot] = {0, 0};
@@ -1103,7 +1169,12 @@ int64_t rhpdhg_batch_launch_count(const rhpdhg_batch *b) { return b ? b->launche
 
 void rhpdhg_batch_free(rhpdhg_batch *b) {
   if (!b) return;
+  if (b->st) cudaStreamSynchronize(b->st);
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
+  if (b->staged) cudaEventDestroy(b->staged);
+  if (b->h_stage) cudaFreeHost(b->h_stage);
+  if (b->h_out) cudaFreeHost(b->h_out);
+  rh::buf_release(b->d_out);
   cudaFree(b->arena);
   cudaFree(b->d_desc);
   cudaFree(b->d_ctls);
