@@ -87,7 +87,7 @@ struct SideLayout {
   int tile_mult = 1;         // consecutive short tiles per work item (1 .. kMaxTileMult)
   int walk = 0;              // instantiation of the ordinary mixed kernels' walk (kWalk*)
   int cta_warps = kBlockWarps;  // warps per CTA of this side's iteration kernels (host only)
-  int wide_rows = 0;         // reported: skewed tiles (wide_rows_pay in setup.cu)
+  int wide_rows = 0;         // skewed tiles (wide_rows_pay in setup.cu): see tile_rows_wide
   int n_tile_groups = 0;     // ceil(n_short_tiles / tile_mult)
   __host__ __device__ int total_items() const { return n_chunks + n_tile_groups; }
 };
@@ -862,6 +862,74 @@ __device__ __forceinline__ void walk_chunk(const SideLayout &lay, const SideVals
   }
 }
 
+// Ordered FP64 tiles (ORD, kOrdered): every product rounded on its own and a row's products added in
+// the order that mixed-precision handles are defined by.  Their restart iterations round FP64
+// anchors' products to FP32, where a last bit decides, and a changed bit there moves an
+// unconverged objective by more than 1e-9.  They run in one iteration of some hundred; FP64 handles,
+// whose sums agree to FP64 rounding in any order, take the cheaper groups of four.
+constexpr bool kOrdered = true;
+
+// Ordered FP64 tiles (see kOrdered) of a skewed side: rows longer than a threshold T are summed by
+// the whole warp (lane-strided partial sums and a shuffle tree, about
+// len/32 + 5 adds per row), the rest lane per row as in tile_rows.  T is the candidate among 8,
+// 16, 32 and the longest row that minimises the warp's FP64 adds, 4 ceil(T / 4) + the sum over
+// rows longer than T of (ceil(len / 32) + 5) (one warp reduction per candidate); a tile whose rows
+// have at most 16 entries keeps T = its longest row.  Rows at or below T are summed exactly as
+// tile_rows sums them. Used only where the same
+// cost model, evaluated over all tiles at set-up, saves FP64 adds (SideLayout::wide_rows).
+template <typename Epi>
+__device__ __forceinline__ void tile_rows_wide(const double *smem, int row0, int nr, int rb,
+                                               int re, int seg_b, uint32_t lm, Epi &epi) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const bool act = lane < nr && !((lm >> lane) & 1u);
+  const int len = act ? re - rb : 0;           // at most kShortMax
+  const int mx = (int)__reduce_max_sync(full, (unsigned)len);
+  int T = mx;
+  if (mx > 16) {
+    int best = (mx + 3) & ~3;
+    const int wadds = ((len + 31) >> 5) + 5;   // this row's adds when summed by the warp
+#pragma unroll
+    for (int c = 8; c <= 32; c *= 2) {
+      if (c >= mx) break;
+      const int cost = c + (int)__reduce_add_sync(full, len > c ? (unsigned)wadds : 0u);
+      if (cost < best) {
+        best = cost;
+        T = c;
+      }
+    }
+  }
+  double dot = 0.0;
+  if (act && len <= T) {
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+    int p = rb - seg_b;
+    const int pe = re - seg_b;
+    for (; p + 4 <= pe; p += 4) {
+      s0 += smem[p];
+      s1 += smem[p + 1];
+      s2 += smem[p + 2];
+      s3 += smem[p + 3];
+    }
+    if (p < pe) s0 += smem[p];
+    if (p + 1 < pe) s1 += smem[p + 1];
+    if (p + 2 < pe) s2 += smem[p + 2];
+    dot = (s0 + s1) + (s2 + s3);
+  }
+  unsigned big = __ballot_sync(full, act && len > T);
+  while (big) {
+    const int r = __ffs(big) - 1;
+    big &= big - 1;
+    const int b = __shfl_sync(full, rb, r) - seg_b, e = __shfl_sync(full, re, r) - seg_b;
+    double s = 0.0;
+    for (int p = b + lane; p < e; p += 32) s += smem[p];
+    s = warp_sum(s);
+    if (lane == r) dot = s;
+  }
+  // one converged epilogue pass (split into the short rows' and the long rows' lanes, the FP64
+  // epilogue issued twice and measured slower)
+  if (act) epi(row0 + lane, dot, false);
+}
+
 // Sums the rows of a short tile from the staged products smem[0, ...) (staged from seg_b on) and
 // runs their epilogues, lane r row r (rows marked long in lm are skipped), each lane going on to its
 // epilogue as soon as its row is summed, so that its loads overlap the other lanes' sums.
@@ -871,15 +939,23 @@ __device__ __forceinline__ void walk_chunk(const SideLayout &lay, const SideVals
 // that stage_segment adds up (one fused multiply-add per entry, every lane busy) leave a quarter
 // of them.  Per FP64 iteration, with warp_reduce_slots, against runs of entries balanced over the
 // lanes and a tree per slot: 2.5M entries with power-law columns 93 to 75 us, flow LP of 30M entries
-// 702 to 621 us, 150k even entries 32 to 21 us.  FP32: four interleaved accumulators.
-template <typename PT, typename Epi>
+// 702 to 621 us, 150k even entries 32 to 21 us.  FP32 and ordered FP64 tiles: four interleaved
+// accumulators.
+template <typename PT, bool ORD, typename Epi>
 __device__ __forceinline__ void tile_rows(const PT *smem, int row0, int nr, int rb, int re,
-                                          int seg_b, uint32_t lm, Epi &epi) {
+                                          int seg_b, uint32_t lm, bool wide, Epi &epi) {
+  constexpr bool kGroups = sizeof(PT) == sizeof(double) && !ORD;
+  if constexpr (sizeof(PT) == sizeof(double) && ORD) {
+    if (wide) {
+      tile_rows_wide(smem, row0, nr, rb, re, seg_b, lm, epi);
+      return;
+    }
+  }
   const int lane = threadIdx.x & 31;
   if (lane >= nr || ((lm >> lane) & 1u)) return;
   int p = rb - seg_b;
   const int pe = re - seg_b;
-  if constexpr (sizeof(PT) == sizeof(double)) {
+  if constexpr (kGroups) {
     PT dot = PT(0);
     if (p < pe) {
       int q = p | 3;                         // the group's last entry
@@ -917,10 +993,10 @@ struct NoPrefetch {
 
 // Stage the products of the segment [seg_b, seg_e) (seg_b 4-aligned) in smem[0, ...): lane
 // handles 4-entry groups g = lane, lane + 32, ..., U at a time (more loads in flight per round,
-// more registers).  FP32 products are staged one by one.  FP64 products are added up within their
-// group of four, up to a row's end (a set bit of ends, see row_ends): smem[p] holds, where entry p
+// more registers).  FP32 and ordered FP64 products are staged one by one.  Other FP64 products are
+// added up within their group of four, up to a row's end (a set bit of ends, see row_ends): smem[p] holds, where entry p
 // ends its row or its group, the sum of the row's entries in the group, and nothing elsewhere.
-template <typename VT, typename PT, int U, int CP, typename Src>
+template <typename VT, typename PT, int U, int CP, bool ORD, typename Src>
 __device__ __forceinline__ void stage_segment(const SideLayout &lay, const SideVals<VT> vals,
                                               const Src &src, PT *smem, int seg_b, int seg_e,
                                               const unsigned *ends) {
@@ -950,7 +1026,7 @@ __device__ __forceinline__ void stage_segment(const SideLayout &lay, const SideV
     for (int u = 0; u < kU; ++u) {
       const int g = g0 + u * kWarp + lane;
       if (g < nvec) {
-        if constexpr (sizeof(PT) == sizeof(double)) {
+        if constexpr (sizeof(PT) == sizeof(double) && !ORD) {
           const unsigned end = ends[g >> 3] >> (4 * (g & 7));
           PT acc = vv[u].v[0] * x[u][0];
 #pragma unroll
@@ -987,7 +1063,8 @@ __device__ __forceinline__ void row_end(unsigned *ends, int seg_b, int rb, int r
 
 // One short tile st of walk_tiles (tile_mult == 1): stage its segment, then lane r sums row r
 // and runs its epilogue.
-template <typename VT, typename PT, int U, int CP, typename Src, typename Epi, typename Pre>
+template <typename VT, typename PT, int U, int CP, bool ORD, typename Src, typename Epi,
+          typename Pre>
 __device__ __forceinline__ void walk_tile(const SideLayout &lay, const SideVals<VT> vals,
                                           const Src &src, PT *smem, Epi &epi, const Pre &pre,
                                           int st) {
@@ -1001,14 +1078,14 @@ __device__ __forceinline__ void walk_tile(const SideLayout &lay, const SideVals<
   int re = __shfl_down_sync(0xffffffffu, rb, 1);
   if (lane >= nr - 1) re = seg_e;
   unsigned *ends = nullptr;
-  if constexpr (sizeof(PT) == sizeof(double)) {
+  if constexpr (sizeof(PT) == sizeof(double) && !ORD) {
     ends = row_ends_clear();
     if (lane < nr) row_end(ends, seg_b, rb, re);
     __syncwarp();
   }
-  stage_segment<VT, PT, U, CP>(lay, vals, src, smem, seg_b, seg_e, ends);
+  stage_segment<VT, PT, U, CP, ORD>(lay, vals, src, smem, seg_b, seg_e, ends);
   __syncwarp();
-  tile_rows<PT>(smem, row0, nr, rb, re, seg_b, lay.long_mask[st], epi);
+  tile_rows<PT, ORD>(smem, row0, nr, rb, re, seg_b, lay.long_mask[st], lay.wide_rows != 0, epi);
   __syncwarp();
 }
 
@@ -1016,8 +1093,8 @@ __device__ __forceinline__ void walk_tile(const SideLayout &lay, const SideVals<
 // tile_mult == 1 only (one tile per item, fewer registers); GROUPED = true walks any layout.
 // pre(row) is called by the lane of each short-tile row before the tile's entries are staged,
 // so that what the row's epilogue will read can be requested while the staging round trips run.
-template <typename VT, typename PT, bool GROUPED, int U, int CP, typename Src, typename Epi,
-          typename GroupDone, typename Pre>
+template <typename VT, typename PT, bool GROUPED, int U, int CP, bool ORD, typename Src,
+          typename Epi, typename GroupDone, typename Pre>
 __device__ __forceinline__ void walk_item(const SideLayout &lay, const SideVals<VT> vals,
                                           const Src &src, PT *smem, const WalkScratch ws,
                                           Epi &epi, GroupDone &gdone, const Pre &pre, int item) {
@@ -1025,7 +1102,7 @@ __device__ __forceinline__ void walk_item(const SideLayout &lay, const SideVals<
   if (item < lay.n_chunks) {
     walk_chunk<VT, PT, CP>(lay, vals, src, ws, epi, gdone, item);
   } else if constexpr (!GROUPED) {
-    walk_tile<VT, PT, U, CP>(lay, vals, src, smem, epi, pre, item - lay.n_chunks);
+    walk_tile<VT, PT, U, CP, ORD>(lay, vals, src, smem, epi, pre, item - lay.n_chunks);
   } else {
     // a group of nt <= tile_mult consecutive short tiles, staged as one segment
     const int t0 = (item - lay.n_chunks) * lay.tile_mult;
@@ -1047,7 +1124,7 @@ __device__ __forceinline__ void walk_item(const SideLayout &lay, const SideVals<
     const int seg_b = __shfl_sync(0xffffffffu, rb0, 0);     // 4-aligned
     const int seg_e = __shfl_sync(0xffffffffu, te, nt - 1);
     unsigned *ends = nullptr;
-    if constexpr (sizeof(PT) == sizeof(double)) {
+    if constexpr (sizeof(PT) == sizeof(double) && !ORD) {
       ends = row_ends_clear();
       for (int m = 0; m < nt; ++m) {
         const int row0 = (t0 + m) * kTileRows;
@@ -1060,7 +1137,7 @@ __device__ __forceinline__ void walk_item(const SideLayout &lay, const SideVals<
       }
       __syncwarp();
     }
-    stage_segment<VT, PT, U, CP>(lay, vals, src, smem, seg_b, seg_e, ends);
+    stage_segment<VT, PT, U, CP, ORD>(lay, vals, src, smem, seg_b, seg_e, ends);
     __syncwarp();
 #pragma unroll 1
     for (int m = 0; m < nt; ++m) {
@@ -1071,14 +1148,14 @@ __device__ __forceinline__ void walk_item(const SideLayout &lay, const SideVals<
       const uint32_t lm_m = __shfl_sync(0xffffffffu, lmk, m);
       int re = __shfl_down_sync(0xffffffffu, rb, 1);
       if (lane >= nr - 1) re = te_m;
-      tile_rows<PT>(smem, row0, nr, rb, re, seg_b, lm_m, epi);
+      tile_rows<PT, ORD>(smem, row0, nr, rb, re, seg_b, lm_m, lay.wide_rows != 0, epi);
     }
     __syncwarp();
   }
 }
 
 template <typename VT, typename PT, bool GROUPED = true, int U = kStageUnroll, int CP = 0,
-          typename Src, typename Epi, typename GroupDone, typename Pre = NoPrefetch>
+          bool ORD = false, typename Src, typename Epi, typename GroupDone, typename Pre = NoPrefetch>
 __device__ __forceinline__ void walk_tiles(const SideLayout &lay, const SideVals<VT> vals,
                                            const Src &src, PT *smem, const WalkScratch ws,
                                            Epi &epi, GroupDone &gdone,
@@ -1087,7 +1164,7 @@ __device__ __forceinline__ void walk_tiles(const SideLayout &lay, const SideVals
   const int nwarps = gridDim.x * (blockDim.x >> 5);
   const int total = lay.total_items();
   for (int item = gwarp; item < total; item += nwarps)
-    walk_item<VT, PT, GROUPED, U, CP>(lay, vals, src, smem, ws, epi, gdone, pre, item);
+    walk_item<VT, PT, GROUPED, U, CP, ORD>(lay, vals, src, smem, ws, epi, gdone, pre, item);
 }
 
 }  // namespace rh

@@ -108,14 +108,14 @@ row_iter_mx(double *smem, const SideLayout &lay, const SideVals<double> v64,
     };
     auto gA = [&](int j) { return x0[j]; };
     auto gdoneA = [&](int grp) { store_group(al, smask & 0x40u, wb.group_part, grp); };
-    walk_tiles<double, double>(lay, v64, gA, my64, wa, epiA, gdoneA);
+    walk_tiles<double, double, true, kStageUnroll, 0, kOrdered>(lay, v64, gA, my64, wa, epiA, gdoneA);
     auto epi = [&](int i, double kd, bool lg) {
       if (lg) row_mx_restart<RHO2>(i, kd, v, sigma, m_eq, check, rp, al, a);
       else row_mx_restart<RHO2>(i, kd, v, sigma, m_eq, check, rp, a, a);
     };
     auto gdone = [&](int grp) { store_group(al, smask & ~0x40u, wb.group_part, grp); };
     auto gB = [&](int j) { return dxt64[j]; };
-    walk_tiles<double, double>(lay, v64, gB, my64, wb, epi, gdone);
+    walk_tiles<double, double, true, kStageUnroll, 0, kOrdered>(lay, v64, gB, my64, wb, epi, gdone);
   } else {
     FprSums<3, DFS> fa, fl;   // restart-norm sums of short rows and of long rows
     auto epi = [&](int i, float kd, bool lg) {
@@ -227,7 +227,7 @@ col_iter_mx(double *smem, const SideLayout &lay, const SideVals<double> v64,
       else col_mx_restart<RHO2>(j, kty, v, tau, check, rp, move, a, a);
     };
     auto gA = [&](int i) { return y0[i] + (double)dyt[i]; };
-    walk_tiles<double, double>(lay, v64, gA, my64, wa, epi, gdone);
+    walk_tiles<double, double, true, kStageUnroll, 0, kOrdered>(lay, v64, gA, my64, wa, epi, gdone);
    } else {
     // first iteration of an epoch: K^T (y~ - y0) in FP64 from the exact dyt64 of the row kernel
     auto epi = [&](int j, double ktd, bool lg) {
@@ -235,7 +235,7 @@ col_iter_mx(double *smem, const SideLayout &lay, const SideVals<double> v64,
       else col_mx_first<RHO2>(j, ktd, v, wf, tauf, check, rp, no_upper, a, a);
     };
     auto gA = [&](int i) { return dyt64[i]; };
-    walk_tiles<double, double>(lay, v64, gA, my64, wb, epi, gdone);
+    walk_tiles<double, double, true, kStageUnroll, 0, kOrdered>(lay, v64, gA, my64, wb, epi, gdone);
    }
   } else {
     auto epi = [&](int j, float ktdyt, bool lg) {

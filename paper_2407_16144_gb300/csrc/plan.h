@@ -20,7 +20,7 @@ struct SidePlan {
   long long nnz_s = 0, nnz_l = 0;   // padded lengths of the short and long arrays
   long long maxseg = 0;             // longest segment of one work item's tile group
   int mult = 1;                     // short tiles per work item
-  int wide_rows = 0;                // reported: skewed tiles (wide_rows_pay in setup.cu)
+  int wide_rows = 0;                // skewed tiles (wide_rows_pay in setup.cu)
   // longest segment of a work item's tile group with 1, 2 and 4 tiles per item (-1 where it
   // exceeds the staging budget): the walks the autotuner may choose instead of the rule's
   long long maxseg_mult[3] = {0, -1, -1};

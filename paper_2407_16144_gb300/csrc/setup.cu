@@ -809,8 +809,8 @@ size_t buf_drop_cache() {
   return freed;
 }
 
-// A side is reported as skewed when summing its tiles' longest rows by whole warps would save at
-// least 15% of the FP64 adds of lane-per-row sums.
+// A side is skewed (its ordered FP64 tiles take tile_rows_wide) when summing its tiles' longest rows
+// by whole warps saves at least 15% of the FP64 adds of lane-per-row sums.
 static bool wide_pays(long long plain, long long best) {
   return plain > 0 && (double)best <= 0.85 * (double)plain;
 }
