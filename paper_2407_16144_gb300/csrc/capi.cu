@@ -928,8 +928,8 @@ int rhpdhg_create(const rhpdhg_problem *lp, const rhpdhg_params *params, void *c
     double *tm = nullptr, *tn = nullptr;
     CKT(dalloc(&tm, m));
     CKT(dalloc(&tn, n));
-    compute_scaling(st, m, n, rp, col, val, cp, ridx, cval, P.ruiz_iters, P.pock_chambolle_alpha,
-                    h->D, h->E, tm, tn);
+    compute_scaling(st, m, n, h->nnz, rp, col, val, cp, ridx, cval, P.ruiz_iters,
+                    P.pock_chambolle_alpha, h->D, h->E, tm, tn);
     if (P.pow2_scaling || P.precision == 2) {
       round_pow2(st, m, h->D);
       round_pow2(st, n, h->E);

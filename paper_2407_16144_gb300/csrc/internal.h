@@ -111,7 +111,7 @@ cudaError_t build_transpose(cudaStream_t st, int m, int n, int nnz, const int *r
                             const double *val, int *cp, int *ridx, double *cval);
 // Ruiz (ruiz_iters passes) then Pock-Chambolle (alpha; skipped when alpha < 0): fills D (m),
 // E (n) so that D K E is the scaled matrix.
-void compute_scaling(cudaStream_t st, int m, int n, const int *rp, const int *col,
+void compute_scaling(cudaStream_t st, int m, int n, long long nnz, const int *rp, const int *col,
                      const double *val, const int *cp, const int *ridx, const double *cval,
                      int ruiz_iters, double alpha, double *D, double *E, double *tmp_m,
                      double *tmp_n);

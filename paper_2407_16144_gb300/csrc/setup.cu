@@ -8,6 +8,7 @@
 #include <climits>
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <unordered_map>
 #include <utility>
 #include <vector>
@@ -91,52 +92,102 @@ __global__ void k_gather_csc(int nnz, const int *perm, const int *rows_of, const
   cval[s] = val[p];
 }
 
-// per row r of a CSR side: OP 0 -> max_p |v_p| rs_r cs_{idx_p};  OP 1 -> sum_p (..)^alpha.
-// G consecutive lanes share a row (strided over its entries, then a fixed shuffle tree), so a
-// long power-law row is spread over a lane group instead of running on one thread.
+// One scaling pass of a CSR side: out_r = rs_r / sqrt(stat_r) (rs_r where the row has no nonzero),
+// with stat_r over the row's entries of |v_p| rs_r cs_{idx_p}: OP 0 their maximum, OP 1 their sum, OP
+// 2 the sum of their powers alpha.  G consecutive lanes share a row (strided over its entries, then a
+// fixed shuffle tree); the rows of a CTA with more than kStatLong entries per lane are then taken by
+// the whole CTA, one after the other (a power-law column of 5000 entries kept 16 lanes busy
+// for 125 us).
+//
+// Bound by the FP64 pipe, where an instruction costs the same with one active lane or 32: two
+// multiplications per entry are left, the order of non-negative doubles being that of their bits; few
+// lanes share a row, so that few are past its end; and the square root and division (about 20
+// instructions) run on packed rows, not in the one lane of a group that has the statistic (61 to 77
+// ms for the create below).  Not a reciprocal square root: on matrices of +-1 the factors lie on
+// the ties of the rounding to powers of two, where the last bit decides.  Create, 64 iterations and
+// free, with k_copy_rows: 30M entries 61.1 to 47.4 ms, 2.5M entries 11.4 to 10.0 ms.
+constexpr int kStatLong = 32;
+
+template <int OP>
+struct StatAcc {
+  double s = 0.0;                    // not negative
+  __device__ __forceinline__ void join(double t) {
+    if (OP == 0) s = __double_as_longlong(t) > __double_as_longlong(s) ? t : s;
+    else s += t;
+  }
+  __device__ __forceinline__ void add(double v, double sr, double c, double alpha) {
+    const double a = v * sr * c;
+    join(OP == 2 ? pow(a, alpha) : a);
+  }
+};
+
 template <int OP, int G>
-__global__ void k_side_stat(int nrows, const int *ptr, const int *idx, const double *val,
-                            const double *rs, const double *cs, double alpha, double *out) {
-  const long long gid = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / G;
-  const int sub = threadIdx.x % G;
-  const bool in = gid < nrows;
-  const int r = in ? (int)gid : 0;
-  double acc = 0.0;
-  if (in) {
-    const double sr = rs[r];
-    const int pe = ptr[r + 1];
+__global__ void __launch_bounds__(256)
+k_side_scale(int nrows, const int *__restrict__ ptr, const int *__restrict__ idx,
+             const double *__restrict__ val, const double *__restrict__ rs,
+             const double *__restrict__ cs, double alpha, double *__restrict__ out) {
+  constexpr int kRows = 256 / G;               // rows of a CTA
+  __shared__ int longs[kRows], nlong;
+  __shared__ double part[8], stat[kRows];
+  if (threadIdx.x == 0) nlong = 0;
+  __syncthreads();
+  const long long r0 = (long long)blockIdx.x * kRows;
+  const int mine = threadIdx.x / G, sub = threadIdx.x % G;
+  const bool in = r0 + mine < nrows;
+  const int r = in ? (int)(r0 + mine) : 0;
+  const int pb = in ? ptr[r] : 0, pe = in ? ptr[r + 1] : 0;
+  const double sr = in ? rs[r] : 0.0;
+  // (a sum keeps one order, that of its G lanes: its last bits reach mixed-precision results)
+  const bool lg = OP == 0 && pe - pb > kStatLong * G;
+  StatAcc<OP> acc;
+  if (!lg) {
 #pragma unroll 4
-    for (int p = ptr[r] + sub; p < pe; p += G) {
-      const double a = fabs(val[p]) * sr * cs[idx[p]];
-      if (OP == 0) acc = fmax(acc, a);
-      else acc += (alpha == 1.0) ? a : pow(a, alpha);
-    }
+    for (int p = pb + sub; p < pe; p += G) acc.add(fabs(val[p]), sr, cs[idx[p]], alpha);
   }
 #pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1) {
-    const double t = __shfl_xor_sync(0xffffffffu, acc, o, G);
-    acc = (OP == 0) ? fmax(acc, t) : acc + t;
+  for (int o = G / 2; o > 0; o >>= 1) acc.join(__shfl_xor_sync(0xffffffffu, acc.s, o, G));
+  if (sub == 0) {
+    if (lg) longs[atomicAdd(&nlong, 1)] = mine;
+    else stat[mine] = acc.s;
   }
-  if (in && sub == 0) out[r] = acc;
+  __syncthreads();
+  for (int k = 0; k < nlong; ++k) {            // the same order of additions whatever the list's
+    const int q = (int)r0 + longs[k];
+    const double sq = rs[q];
+    const int qe = ptr[q + 1];
+    StatAcc<OP> a;
+#pragma unroll 4
+    for (int p = ptr[q] + threadIdx.x; p < qe; p += 256) a.add(fabs(val[p]), sq, cs[idx[p]], alpha);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a.join(__shfl_xor_sync(0xffffffffu, a.s, o));
+    if (threadIdx.x % 32 == 0) part[threadIdx.x / 32] = a.s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < 8; ++w) a.join(part[w]);
+      stat[longs[k]] = a.s;
+    }
+    __syncthreads();
+  }
+  const int t = threadIdx.x;
+  if (t < kRows && r0 + t < nrows) {
+    const double s = stat[t], f = rs[r0 + t];
+    out[r0 + t] = s > 0.0 ? f / sqrt(s) : f;
+  }
 }
 
-__global__ void k_scale_update(int n, const double *stat, double *scale) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double s = stat[i];
-  if (s > 0.0) scale[i] = scale[i] / sqrt(s);
-}
-
-// copy each row's entries, scaled, to its place in the short or long arrays (warp per row),
-// with an FP32 (LOWP 1) or BF16 (LOWP 2) copy of the scaled values
-template <int LOWP>
-__global__ void k_copy_rows(int nrows, const int *ptr, const int *idx, const double *val,
-                            const double *rs, const double *cs, const int *dst,
-                            const uint32_t *long_mask, int *idx_s, double *val_s, float *val32_s,
-                            __nv_bfloat16 *val16_s, int *idx_l, double *val_l, float *val32_l,
-                            __nv_bfloat16 *val16_l) {
-  const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
+// copy each row's entries, scaled, to its place in the short or long arrays (G lanes per row: a
+// warp per row left most lanes idle on rows of a few entries), with an FP32
+// (LOWP 1) or BF16 (LOWP 2) copy of the scaled values
+template <int LOWP, int G>
+__global__ void __launch_bounds__(256)
+k_copy_rows(int nrows, const int *__restrict__ ptr, const int *__restrict__ idx,
+            const double *__restrict__ val, const double *__restrict__ rs,
+            const double *__restrict__ cs, const int *__restrict__ dst,
+            const uint32_t *__restrict__ long_mask, int *idx_s, double *val_s, float *val32_s,
+            __nv_bfloat16 *val16_s, int *idx_l, double *val_l, float *val32_l,
+            __nv_bfloat16 *val16_l) {
+  const long long w = (blockIdx.x * 256LL + threadIdx.x) / G;
+  const int lane = threadIdx.x % G;
   if (w >= nrows) return;
   const int r = (int)w;
   const bool lg = (long_mask[r >> 5] >> (r & 31)) & 1u;
@@ -146,7 +197,8 @@ __global__ void k_copy_rows(int nrows, const int *ptr, const int *idx, const dou
   __nv_bfloat16 *vh = lg ? val16_l : val16_s;
   const int b = ptr[r], e = ptr[r + 1], o = dst[r];
   const double sr = rs[r];
-  for (int p = b + lane; p < e; p += 32) {
+#pragma unroll 4
+  for (int p = b + lane; p < e; p += G) {
     const int j = idx[p];
     const double v = sr * val[p] * cs[j];
     ix[o + (p - b)] = j;
@@ -215,7 +267,13 @@ __global__ void k_fill(int n, T v, T *x) {
 
 __global__ void k_vmul(int n, const double *a, const double *x, double *y, int div) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) y[i] = div ? x[i] / a[i] : a[i] * x[i];
+  if (i >= n) return;
+  const double v = x[i];
+  // 0 and +-inf divided by a positive factor are themselves (bounds, mostly; a division takes
+  // about ten FP64 instructions)
+  const long long b = __double_as_longlong(v) & 0x7fffffffffffffffll;
+  if (!div) y[i] = a[i] * v;
+  else y[i] = b == 0 || b == 0x7ff0000000000000ll ? v : v / a[i];
 }
 
 __global__ void k_vclamp(int n, double *x, const double *l, const double *u) {
@@ -614,57 +672,73 @@ done:
   return err;
 }
 
-// lanes per row for a side with `nnz` entries over `nrows` rows (the mean row length, rounded
-// up to a power of two, 4 to 32)
-static int stat_group(long long nnz, int nrows) {
+// f(std::integral_constant<int, G>) for a side's lanes per row, which decide only the time: an
+// eighth of the mean row length, at least kMin (1 or 4) and at most 32.  More lanes leave more of
+// them idle past the rows' ends (17 entries take 5 steps of 4 lanes, 85% busy, or one and a bit of
+// 16); fewer than four do not read whole sectors, which only pays where rows have about as few entries.
+template <int kMin, class F>
+static void with_group(long long nnz, int nrows, F &&f) {
   const double mean = nrows > 0 ? (double)nnz / nrows : 0.0;
-  int g = 4;
-  while (g < 32 && g < mean) g *= 2;
-  return g;
+  if (kMin == 1 && mean <= 4.0) f(std::integral_constant<int, kMin>{});
+  else if (mean <= 32.0) f(std::integral_constant<int, 4>{});
+  else if (mean <= 64.0) f(std::integral_constant<int, 8>{});
+  else if (mean <= 128.0) f(std::integral_constant<int, 16>{});
+  else f(std::integral_constant<int, 32>{});
+}
+// The same for sums, whose order they decide: the mean row length rounded up to a power of two.
+template <class F>
+static void with_sum_group(long long nnz, int nrows, F &&f) {
+  const double mean = nrows > 0 ? (double)nnz / nrows : 0.0;
+  if (mean <= 4.0) f(std::integral_constant<int, 4>{});
+  else if (mean <= 8.0) f(std::integral_constant<int, 8>{});
+  else if (mean <= 16.0) f(std::integral_constant<int, 16>{});
+  else f(std::integral_constant<int, 32>{});
 }
 
 template <int OP>
-static void side_stat(cudaStream_t st, int nrows, long long nnz, const int *ptr, const int *idx,
-                      const double *val, const double *rs, const double *cs, double alpha,
-                      double *out) {
-  const int g = stat_group(nnz, nrows);
-  const long long threads = (long long)nrows * g;
-  const int nb = (int)((threads + 255) / 256);
-  if (nb <= 0) return;
-  switch (g) {
-    case 4: k_side_stat<OP, 4><<<nb, 256, 0, st>>>(nrows, ptr, idx, val, rs, cs, alpha, out); break;
-    case 8: k_side_stat<OP, 8><<<nb, 256, 0, st>>>(nrows, ptr, idx, val, rs, cs, alpha, out); break;
-    case 16: k_side_stat<OP, 16><<<nb, 256, 0, st>>>(nrows, ptr, idx, val, rs, cs, alpha, out); break;
-    default: k_side_stat<OP, 32><<<nb, 256, 0, st>>>(nrows, ptr, idx, val, rs, cs, alpha, out); break;
-  }
+static void side_scale(cudaStream_t st, int nrows, long long nnz, const int *ptr, const int *idx,
+                       const double *val, const double *rs, const double *cs, double alpha,
+                       double *out) {
+  if (nrows <= 0) return;
+  auto pass = [&](auto G) {
+    k_side_scale<OP, G()><<<nblocks((long long)nrows * G(), 256), 256, 0, st>>>(
+        nrows, ptr, idx, val, rs, cs, alpha, out);
+  };
+  if (OP == 0) with_group<1>(nnz, nrows, pass);
+  else with_sum_group(nnz, nrows, pass);
+  count_launches(1);
 }
 
-void compute_scaling(cudaStream_t st, int m, int n, const int *rp, const int *col,
+void compute_scaling(cudaStream_t st, int m, int n, long long nnz, const int *rp, const int *col,
                      const double *val, const int *cp, const int *ridx, const double *cval,
                      int ruiz_iters, double alpha, double *D, double *E, double *tmp_m,
                      double *tmp_n) {
-  long long nnz = 0;
-  {
-    int last = 0;
-    if (m > 0) cudaMemcpyAsync(&last, rp + m, sizeof(int), cudaMemcpyDeviceToHost, st);
-    cudaStreamSynchronize(st);
-    nnz = last;
+  // both sides' new factors from the same current ones, so every pass goes from one pair of
+  // buffers to the other; the last lands in D, E
+  const int passes = ruiz_iters + (alpha >= 0.0 ? 1 : 0);
+  if (passes % 2) {
+    std::swap(D, tmp_m);
+    std::swap(E, tmp_n);
   }
   k_fill<<<nblocks(m, 256), 256, 0, st>>>(m, 1.0, D);
   k_fill<<<nblocks(n, 256), 256, 0, st>>>(n, 1.0, E);
-  count_launches(2 + 4LL * ruiz_iters + (alpha >= 0.0 ? 4 : 0));
-  for (int it = 0; it < ruiz_iters; ++it) {
-    // both norms from the same current matrix, then both updates
-    side_stat<0>(st, m, nnz, rp, col, val, D, E, 1.0, tmp_m);
-    side_stat<0>(st, n, nnz, cp, ridx, cval, E, D, 1.0, tmp_n);
-    k_scale_update<<<nblocks(m, 256), 256, 0, st>>>(m, tmp_m, D);
-    k_scale_update<<<nblocks(n, 256), 256, 0, st>>>(n, tmp_n, E);
-  }
-  if (alpha >= 0.0) {
-    side_stat<1>(st, m, nnz, rp, col, val, D, E, alpha, tmp_m);
-    side_stat<1>(st, n, nnz, cp, ridx, cval, E, D, 2.0 - alpha, tmp_n);
-    k_scale_update<<<nblocks(m, 256), 256, 0, st>>>(m, tmp_m, D);
-    k_scale_update<<<nblocks(n, 256), 256, 0, st>>>(n, tmp_n, E);
+  count_launches(2);
+  for (int it = 0; it < passes; ++it) {
+    if (it < ruiz_iters) {
+      side_scale<0>(st, m, nnz, rp, col, val, D, E, 1.0, tmp_m);
+      side_scale<0>(st, n, nnz, cp, ridx, cval, E, D, 1.0, tmp_n);
+    } else {
+      auto pock_chambolle = [&](auto OP, auto OQ) {
+        side_scale<OP()>(st, m, nnz, rp, col, val, D, E, alpha, tmp_m);
+        side_scale<OQ()>(st, n, nnz, cp, ridx, cval, E, D, 2.0 - alpha, tmp_n);
+      };
+      using One = std::integral_constant<int, 1>;
+      using Pow = std::integral_constant<int, 2>;
+      if (alpha == 1.0) pock_chambolle(One{}, One{});
+      else pock_chambolle(Pow{}, Pow{});
+    }
+    std::swap(D, tmp_m);
+    std::swap(E, tmp_n);
   }
 }
 
@@ -936,7 +1010,6 @@ bool plan_side(const int *hp, int nrows, SidePlan *p) {
 cudaError_t build_side(cudaStream_t st, int nrows, int nnz, const int *ptr, const int *idx,
                        const double *val, const double *rscale, const double *cscale,
                        int lowp, SideStore *out) {
-  (void)nnz;
   SideStore s;
   cudaError_t err = cudaSuccess;
   const int ntiles = (int)(((long long)nrows + kTileRows - 1) / kTileRows);
@@ -1036,15 +1109,16 @@ cudaError_t build_side(cudaStream_t st, int nrows, int nnz, const int *ptr, cons
     TRY(cudaMemsetAsync(s.val16_l, 0, nnz_l * sizeof(__nv_bfloat16), st));
   }
   if (nrows > 0) {
-    const int nb = nblocks((long long)nrows * 32, 256);
-    auto copy = [&](auto kern) {
-      kern<<<nb, 256, 0, st>>>(nrows, ptr, idx, val, rscale, cscale, d_dst, s.long_mask,
-                               s.idx_s, s.val64_s, s.val32_s, s.val16_s, s.idx_l, s.val64_l,
-                               s.val32_l, s.val16_l);
-    };
-    if (lowp == 1) copy(k_copy_rows<1>);
-    else if (lowp == 2) copy(k_copy_rows<2>);
-    else copy(k_copy_rows<0>);
+    with_group<4>(nnz, nrows, [&](auto G) {
+      auto copy = [&](auto kern) {
+        kern<<<nblocks((long long)nrows * G(), 256), 256, 0, st>>>(
+            nrows, ptr, idx, val, rscale, cscale, d_dst, s.long_mask, s.idx_s, s.val64_s,
+            s.val32_s, s.val16_s, s.idx_l, s.val64_l, s.val32_l, s.val16_l);
+      };
+      if (lowp == 1) copy(k_copy_rows<1, G()>);
+      else if (lowp == 2) copy(k_copy_rows<2, G()>);
+      else copy(k_copy_rows<0, G()>);
+    });
     count_launches(1);
   }
   // ---- walk scratch ------------------------------------------------------------------------
