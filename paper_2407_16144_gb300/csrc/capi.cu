@@ -1135,11 +1135,11 @@ int rhpdhg_create(const rhpdhg_problem *lp, const rhpdhg_params *params, void *c
                      h->certx, h->dxt64, h->c, h->l, h->u, h->E, h->Einv, h->certx2, h->act};
   algorithmic_bytes(h);
   {
-    // the ordinary mixed kernels read the matrix stream evict-first where one iteration's
-    // bytes exceed L2 (see Vec4 in common.cuh)
+    // where one iteration's bytes exceed L2 the ordinary mixed kernels read the matrix stream
+    // evict-first (see Vec4 in common.cuh) and the FP64 kernels prefetch their epilogues' rows
     int l2 = 0;
     CKC(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, h->dev));
-    h->ic.l2_first = h->mixed && h->bytes_row + h->bytes_col > (double)l2 ? 1 : 0;
+    h->ic.l2_first = h->bytes_row + h->bytes_col > (double)l2 ? 1 : 0;
   }
   h->launches = launches_so_far() - launches0;
   CKC(cudaStreamSynchronize(st));

@@ -205,8 +205,9 @@ struct IterConsts {
   int df_sums;                // mixed: 1 = double-float restart-norm sums from the lane up,
                               // 0 = FP32 sums at every level
   int adaptive;               // 1 = adaptive step rule (inadmissible steps are redone)
-  int l2_first;               // mixed: 1 = the ordinary kernels read the matrix stream with the
-                              // L2 evict-first policy (one iteration's bytes exceed L2)
+  int l2_first;               // 1 = one iteration's bytes exceed L2: the ordinary mixed kernels
+                              // read the matrix stream with the L2 evict-first policy, the FP64
+                              // kernels prefetch what their epilogues read
 };
 
 // ---------------------------------------------------------------------------------------------
