@@ -28,8 +28,8 @@ constexpr int kKktSlots = kKktSlotCount;   // stride of a block's partials
 constexpr int kKktUsed = 7;                // 0 rp2, 1 qy, 2 qq, 3 rd2, 4 cx, 5 bnd, 6 cc
 constexpr int kKktRowSlots = 3;            // the first three come from the row kernel
 constexpr int kKktFlag = 5;                // dout[5]: 1 if the CSR held an index out of range
-constexpr int kKktStage = 704;             // entries a warp stages at a time (22 per row of 32)
-constexpr int kKktUnroll = 4;              // entries per lane in flight
+constexpr int kKktStage = 704;             // entries a warp stages at a time (22 per row of 32): a
+                                           // multiple of 4
 constexpr int kKktRowCtas = 4;             // resident CTAs per SM of the row kernel (45 KB each)
 
 __device__ __forceinline__ double block_sum(double v, double *sh) {
@@ -44,77 +44,16 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
   return r;   // valid in thread 0
 }
 
-// Row sums of one warp's staged segment s[0, len), balanced over the lanes: returns, in lane r, the
-// sum of s[b, e) (b, e: that lane's row, 0 <= b <= e <= len; rows in lane order without overlap,
-// so the rows that are not empty tile [b of the first, e of the last)).  The segment's contents are
-// consumed.
-//
-// What bounds it is the FP64 pipe, which is narrow on this part and issues a warp's add as slowly
-// for one active lane as for 32: one lane per row costs the longest row's adds.  Here every lane
-// adds an equal run of L consecutive entries (L odd: no shared-memory bank conflicts), writing its
-// running sum over the last entry of every row, and of the run, that it completes; lane r then adds
-// the one or few partial sums of its row, in entry order.  That is L + (runs a row spans) adds for
-// the warp.  Where no row is longer than that, one lane per row is kept.
-template <typename PT>
-__device__ __forceinline__ PT balanced_row_sum(PT *s, int len, int b, int e) {
-  const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  const int mx = (int)__reduce_max_sync(full, (unsigned)(e - b));
-  const int L = ((len + kWarp - 1) / kWarp) | 1;
-  if (mx <= L + (mx + L - 2) / L) {
-    PT t = PT(0);
-#pragma unroll 4
-    for (int p = b; p < e; ++p) t += s[p];
-    return t;
-  }
-  // the row that holds this lane's first entry: the number of rows that end at or before it
-  const int start = lane * L, stop = min(start + L, len);
-  int r = 0;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-    if (__shfl_sync(full, e, r + o - 1) <= start) r += o;
-  const unsigned some = __ballot_sync(full, e > b);
-  int end = __shfl_sync(full, e, r);
-  PT acc = PT(0);
-#pragma unroll 4
-  for (int i = 0; i < L; ++i) {
-    const int p = start + i;
-    const bool in = p < stop;
-    if (in) acc += s[p];
-    const bool done = p + 1 == end;
-    if (in && (done || i == L - 1)) s[p] = acc;
-    if (done) {
-      acc = PT(0);
-      const unsigned rest = some & ~((2u << r) - 1u);   // the next row that is not empty
-      r = rest ? __ffs((int)rest) - 1 : r;
-    }
-    end = __shfl_sync(full, e, r);
-  }
-  __syncwarp();
-  PT t = PT(0);
-  if (e > b) {
-    // run of an entry by a multiplication: exact for entries below 1056 and L up to 33
-    static_assert(kSegBudget <= 1024, "entries of a staged segment");
-    const unsigned inv = (65536u + (unsigned)L - 1u) / (unsigned)L;
-    int c = (int)(((unsigned)b * inv) >> 16);
-    const int c1 = (int)(((unsigned)(e - 1) * inv) >> 16);
-    t = s[min((c + 1) * L, e) - 1];
-    while (c < c1) {
-      ++c;
-      t += s[min((c + 1) * L, e) - 1];
-    }
-  }
-  return t;
-}
-
 // One warp takes 32 consecutive rows: their entries are read as one contiguous segment, kKktStage at
-// a time, every lane on consecutive entries (one thread per row read 12 bytes here and 12 bytes
-// 200 bytes further on).  Each entry finds its row among the 32 row ends by a search in shuffles,
-// scatters val * y_row and stages val * x_j in shared memory, from which the rows are summed
-// balanced over the lanes (balanced_row_sum).  Bound by the FP64 pipe (62% busy; two products and
-// one sum per entry) and the scattered FP64 additions in L2: 280 us for 30M entries.  The whole
-// evaluation of that LP took 950 us with a thread per row, a cudaMalloc and cudaFree per call and
-// floating-point comparisons in the column kernel, and takes 464 us.
+// a time, a lane on four consecutive entries (one thread per row read 12 bytes here and 12 bytes
+// 200 bytes further on).  The lane finds its first entry's row among the 32 row ends by a search in
+// shuffles and follows the ends through the bits of row_ends; it scatters val * y_row and adds
+// val * x_j up within its four entries and the row, as stage_segment does, so that a row's sum is
+// left with a quarter of its additions.  Bound by the FP64 pipe (a multiplication and a fused
+// multiply-add per entry) and the scattered FP64 additions in L2.  The evaluation of a 30M-entry
+// LP took 950 us with a thread per row, a cudaMalloc and cudaFree per call and floating-point
+// comparisons in the column kernel, 464 us with runs of entries balanced over the lanes, and takes
+// 407 us.
 //
 // Rows whose offsets fall outside [0, nnz] or decrease, and entries whose column lies outside
 // [0, n), are skipped and reported through flag (the caller's CSR is not validated beforehand);
@@ -156,38 +95,56 @@ k_kkt_rows(int m, int m_eq, int n, long long nnz, const long long *__restrict__ 
         const int len = (int)min((long long)kKktStage, seg_e - base);
         const int lo = (int)min(max(p0 - base, 0ll), (long long)len);
         const int hi = (int)min(max(p1 - base, 0ll), (long long)len);
-        for (int o = 0; o < len; o += 32 * kKktUnroll) {
-          int j[kKktUnroll];
-          double v[kKktUnroll], xj[kKktUnroll];
+        unsigned *ends = row_ends_clear();
+        row_end(ends, 0, lo, hi);
+        const unsigned some = __ballot_sync(full, hi > lo);
+        __syncwarp();
+        for (int o = 4 * lane; o - 4 * lane < len; o += 32 * 4) {
+          int j[4];
+          double v[4], xj[4];
 #pragma unroll
-          for (int u = 0; u < kKktUnroll; ++u) {
-            const int k = o + 32 * u + lane;
-            j[u] = k < len ? col[base + k] : 0;
-            v[u] = k < len ? val[base + k] : 0.0;
+          for (int u = 0; u < 4; ++u) {
+            j[u] = o + u < len ? col[base + o + u] : 0;
+            v[u] = o + u < len ? val[base + o + u] : 0.0;
           }
 #pragma unroll
-          for (int u = 0; u < kKktUnroll; ++u) {
+          for (int u = 0; u < 4; ++u) {
             const bool ok = j[u] >= 0 && j[u] < n;
             if (!ok) *flag = 1.0;
-            xj[u] = ok && o + 32 * u + lane < len ? x[j[u]] : 0.0;
+            xj[u] = ok && o + u < len ? x[j[u]] : 0.0;
+            if (!ok) v[u] = 0.0;
           }
+          int r = 0;                         // rows that end at or before entry o
 #pragma unroll
-          for (int u = 0; u < kKktUnroll; ++u) {
-            const int k = o + 32 * u + lane;
-            int r = 0;                       // rows that end at or before entry k
+          for (int h = 16; h > 0; h >>= 1)
+            if (__shfl_sync(full, hi, r + h - 1) <= o) r += h;
+          const unsigned end = o < len ? ends[o >> 5] >> (o & 31) : 0u;
+          double acc = 0.0;
 #pragma unroll
-            for (int h = 16; h > 0; h >>= 1)
-              if (__shfl_sync(full, hi, r + h - 1) <= k) r += h;
+          for (int u = 0; u < 4; ++u) {
             const double yr = __shfl_sync(full, yi, r);
-            if (k < len) {
-              const bool ok = j[u] >= 0 && j[u] < n;
-              st[k] = ok ? v[u] * xj[u] : 0.0;
-              if (ok) atomicAdd(kty + j[u], v[u] * yr);
+            if (o + u < len && j[u] >= 0 && j[u] < n) atomicAdd(kty + j[u], v[u] * yr);
+            acc = fma(v[u], xj[u], acc);
+            if ((end >> u) & 1u) {
+              st[o + u] = acc;
+              acc = 0.0;
+              const unsigned rest = some & ~((2u << r) - 1u);    // the next row that is not empty
+              r = rest ? __ffs((int)rest) - 1 : r;
+            } else if (u == 3 && o < len) {
+              st[o + 3] = acc;
             }
+            __syncwarp();
           }
         }
         __syncwarp();
-        kx += balanced_row_sum(st, len, lo, hi);
+        if (lo < hi) {
+          int q = lo | 3;                    // the last entry of the row's first four
+          kx += st[min(q, hi - 1)];
+          while (q < hi - 1) {
+            q += 4;
+            kx += st[min(q, hi - 1)];
+          }
+        }
         __syncwarp();
       }
     }
