@@ -198,9 +198,11 @@ __device__ void rows_stat(int nrows, const int *ptr, const int *idx, const doubl
     if (r < nrows) {
       const double sr = rs[r];
       for (int p = ptr[r] + gl; p < ptr[r + 1]; p += g) {
-        const double a = fabs(val[p]) * sr * cs[idx[p]];
+        // (not fused with the sum, whatever the context compiles to: the factors' last bits reach a
+        // mixed slot's FP32 values)
+        const double a = __dmul_rn(__dmul_rn(fabs(val[p]), sr), cs[idx[p]]);
         if (OP == 0) s = fmax(s, a);
-        else s += (alpha == 1.0) ? a : pow(a, alpha);
+        else s = __dadd_rn(s, (alpha == 1.0) ? a : pow(a, alpha));
       }
     }
     s = OP == 0 ? group_max(s, g) : group_sum(s, g);
@@ -215,6 +217,15 @@ __device__ void scale_update(int n, const double *stat, double *scale) {
   }
 }
 
+// This thread's part of ||x||^2, in the chains of kChain threads: the norms give the step and the
+// primal weight, whose last bits a mixed slot's results follow, whatever the CTA's width.
+__device__ __forceinline__ double chain_sumsq(int k, const double *x) {
+  double s = 0.0;
+  if (threadIdx.x < kChain)
+    for (int i = threadIdx.x; i < k; i += kChain) s += x[i] * x[i];
+  return s;
+}
+
 // The whole create-time pipeline of one LP, inside its CTA.
 __device__ void batch_setup(const BatchDesc &d, double (*sh)[kMaxPartials]) {
   const int m = d.m, n = d.n;
@@ -225,9 +236,7 @@ __device__ void batch_setup(const BatchDesc &d, double (*sh)[kMaxPartials]) {
   double *q = const_cast<double *>(rvv.q), *c = const_cast<double *>(cvv.c);
   double *l = const_cast<double *>(cvv.l), *u = const_cast<double *>(cvv.u);
   // norms of the unscaled data
-  double a = 0.0, b = 0.0;
-  for (int i = threadIdx.x; i < m; i += kBT) a += q[i] * q[i];
-  for (int j = threadIdx.x; j < n; j += kBT) b += c[j] * c[j];
+  double a = chain_sumsq(m, q), b = chain_sumsq(n, c);
   const double qn = sqrt(block_sum1(a, sh)), cn = sqrt(block_sum1(b, sh));
   // Ruiz then Pock-Chambolle
   for (int i = threadIdx.x; i < m; i += kBT) D[i] = 1.0;
@@ -276,10 +285,8 @@ __device__ void batch_setup(const BatchDesc &d, double (*sh)[kMaxPartials]) {
     Einv[j] = 1.0 / E[j];
   }
   __syncthreads();
-  a = 0.0;
-  b = 0.0;
-  for (int i = threadIdx.x; i < m; i += kBT) a += q[i] * q[i];
-  for (int j = threadIdx.x; j < n; j += kBT) b += c[j] * c[j];
+  a = chain_sumsq(m, q);
+  b = chain_sumsq(n, c);
   const double qhn = sqrt(block_sum1(a, sh)), chn = sqrt(block_sum1(b, sh));
   // power iteration on K^T K from 1/sqrt(n): v in x, K v in kx, K^T K v in kty
   double *v = cvv.x, *um = rvv.kx, *w = cvv.kty;
@@ -296,19 +303,15 @@ __device__ void batch_setup(const BatchDesc &d, double (*sh)[kMaxPartials]) {
       auto g2 = [&](int i) { return um[i]; };
       rows_apply(n, d.cp, d.ri, d.cv, d.gc, g2, f2);
       __syncthreads();
-      double ss = 0.0;
-      for (int j = threadIdx.x; j < n; j += kBT) ss += w[j] * w[j];
-      const double nrm = sqrt(block_sum1(ss, sh)), inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
-      for (int j = threadIdx.x; j < n; j += kBT) v[j] = w[j] * inv;
+      const double nrm = sqrt(block_sum1(chain_sumsq(n, w), sh));
+      for (int j = threadIdx.x; j < n; j += kBT) v[j] = nrm > 0.0 ? w[j] / nrm : 0.0;
       __syncthreads();
     }
     auto f1 = [&](int r, double s) { um[r] = s; };
     auto g1 = [&](int j) { return v[j]; };
     rows_apply(m, d.rp, d.ci, d.rv, d.gr, g1, f1);
     __syncthreads();
-    double ss = 0.0;
-    for (int i = threadIdx.x; i < m; i += kBT) ss += um[i] * um[i];
-    smax = sqrt(block_sum1(ss, sh));
+    smax = sqrt(block_sum1(chain_sumsq(m, um), sh));
   }
   double eta;
   if (d.step_size > 0) eta = d.step_size;
