@@ -74,12 +74,18 @@ __device__ __forceinline__ bool col_defers(const IterConsts &ic, int phase, bool
   return phase == 0 && !check && !cert && !move && !ic.adaptive;
 }
 
+// The Halpern weight after inner iteration k (not read where that iteration restarts).
+__device__ __forceinline__ void halpern_weight(Ctl *ctl, long long k) {
+  ctl->w = (k + 1.0) / (k + 2.0);
+}
+
 // rc: the deferred column stage's sums (dcol; see col_defers), (t, k, n_ep) the iteration after
-// it.
+// it.  weight: false where another warp runs halpern_weight meanwhile (its FP64 division alone takes
+// about 650 clocks).
 __device__ __forceinline__ void row_finalize(Ctl *ctl, const IterConsts &ic, const double *r,
                                              long long t, long long k, long long n_ep,
                                              double sigma, bool move, bool dcol = false,
-                                             const double *rc = nullptr) {
+                                             const double *rc = nullptr, bool weight = true) {
   if (dcol) {
     // the finaliser the column stage left: its sums and the advance of (t, k, n)
     ctl->col_deferred = 0;
@@ -178,7 +184,7 @@ __device__ __forceinline__ void row_finalize(Ctl *ctl, const IterConsts &ic, con
     ctl->k_next = 0;
     ctl->n_next = n_ep + 1;
   } else {
-    ctl->w = (k + 1.0) / (k + 2.0);
+    if (weight) halpern_weight(ctl, k);
     ctl->k_next = k + 1;
     ctl->n_next = n_ep;
   }

@@ -57,7 +57,7 @@ __host__ __device__ constexpr int mx_max_regs(int mode, int walk, int dfs) {
 // MODE 0 is the ordinary (FP32) iteration and returns at once when a restart is pending; MODE 1 is
 // the restart iteration (FP64 walks) and returns at once otherwise.
 // CP: the matrix stream's cache policy of the ordinary kernels' walk (see Vec4 in common.cuh).
-template <int RHO2, int MODE, int WALK, int DFS, int LP, int CP>
+template <int RHO2, int MODE, int WALK, int DFS, int LP, int CP, bool BOTH>
 __device__ __forceinline__ void
 row_iter_mx(double *smem, const SideLayout &lay, const SideVals<double> v64,
             const SideVals<LowT<LP>> v32, const WalkScratch wa, const WalkScratch wb,
@@ -150,7 +150,10 @@ row_iter_mx(double *smem, const SideLayout &lay, const SideVals<double> v64,
     double rc[2] = {0.0, 0.0};
     if (dcol)   // the deferred ordinary column stage's two sums (its packed slots)
       dcol_finish<col_df_slots<0>(), DFS == 1>(dc, pre, rc);
-    if (threadIdx.x == 0) row_finalize(ctl, ic, r, t, k, n_ep, sigma, move, dcol, rc);
+    if (threadIdx.x == 0) row_finalize(ctl, ic, r, t, k, n_ep, sigma, move, dcol, rc, !BOTH);
+    // (small LPs only, 75k entries 13.5 to 13.3 ms in 640 iterations: with 2.5M entries it measured
+    // 1% slower, in the FP64 kernels 2% slower on LPs beyond L2)
+    if (BOTH && threadIdx.x == blockDim.x - kWarp) halpern_weight(ctl, k);
   }
 }
 
@@ -169,13 +172,13 @@ k_row_iter_mx(SideLayout lay, SideVals<double> v64, SideVals<LowT<LP>> v32, Walk
   if (ctl->status != kRunning) return;
   if constexpr (MODE == 2) {
     if (ctl->restart_pending)
-      row_iter_mx<RHO2, 1, kWalkGrouped, 0, LP, 0>(smem, lay, v64, v32, wa, wb, v, dxt, dxt64, x0,
+      row_iter_mx<RHO2, 1, kWalkGrouped, 0, LP, 0, true>(smem, lay, v64, v32, wa, wb, v, dxt, dxt64, x0,
                                                    ctl, part, ic, dc);
     else
-      row_iter_mx<RHO2, 0, WALK, DFS, LP, CP>(smem, lay, v64, v32, wa, wb, v, dxt, dxt64, x0, ctl,
+      row_iter_mx<RHO2, 0, WALK, DFS, LP, CP, true>(smem, lay, v64, v32, wa, wb, v, dxt, dxt64, x0, ctl,
                                               part, ic, dc);
   } else {
-    row_iter_mx<RHO2, MODE, WALK, DFS, LP, CP>(smem, lay, v64, v32, wa, wb, v, dxt, dxt64, x0, ctl,
+    row_iter_mx<RHO2, MODE, WALK, DFS, LP, CP, false>(smem, lay, v64, v32, wa, wb, v, dxt, dxt64, x0, ctl,
                                                part, ic, dc);
   }
 }
