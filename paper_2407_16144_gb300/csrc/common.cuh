@@ -315,17 +315,6 @@ __device__ __forceinline__ DF df_prod(float a, float b) {
   return r;
 }
 
-__device__ __forceinline__ DF df_warp_sum(DF v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    DF w;
-    w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
-    w.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
-    v = df_add(v, w);
-  }
-  return v;
-}
-
 // The packed slots carry either double-floats (EXACT) or plain FP32 sums in hi (lo = 0), which
 // the same reductions add with single FP32 additions: the FP32 option of the mixed-precision
 // restart-norm sums, whose dependent chains in the grid reduction stay short.
@@ -333,11 +322,6 @@ template <bool EXACT>
 __device__ __forceinline__ DF dfx_add(DF x, DF y) {
   if constexpr (EXACT) return df_add(x, y);
   else return DF{__fadd_rn(x.hi, y.hi), 0.f};
-}
-template <bool EXACT>
-__device__ __forceinline__ DF dfx_warp_sum(DF v) {
-  if constexpr (EXACT) return df_warp_sum(v);
-  else return DF{warp_sum(v.hi), 0.f};
 }
 
 // A double-float travels through the 8-byte partial slots bit-packed (no FP64 arithmetic).
