@@ -111,6 +111,13 @@ void finish_request(rhpdhg_server *s, Request &r, const rhpdhg_result &res) {
   s->completed++;
 }
 
+// Result of a request whose poll failed: no solved status without its vectors.
+rhpdhg_result failed_result() {
+  rhpdhg_result res{};
+  res.status = RHPDHG_STATUS_NUMERICAL_ERROR;
+  return res;
+}
+
 void worker_loop(rhpdhg_server *s) {
   cudaSetDevice(s->dev);
   while (!s->stop.load()) {
@@ -155,9 +162,7 @@ void worker_loop(rhpdhg_server *s) {
               admitted = true;
             } else {
               if (h) rhpdhg_free(h);
-              rhpdhg_result res{};
-              res.status = RHPDHG_STATUS_NUMERICAL_ERROR;
-              finish_request(s, r, res);
+              finish_request(s, r, failed_result());
               it = s->pending.erase(it);
               continue;
             }
@@ -205,7 +210,10 @@ void worker_loop(rhpdhg_server *s) {
         if (st == RHPDHG_STATUS_RUNNING) {
           res.status = RHPDHG_STATUS_CANCELLED;
         } else {
-          rhpdhg_batch_poll(s->batch, r.slot, &res);
+          const int rc = rhpdhg_batch_poll(s->batch, r.slot, &res);
+          // out of memory: the slot keeps its result and is polled again in the next turn
+          if (rc == RHPDHG_ERR_OOM && !r.cancel) continue;
+          if (rc != RHPDHG_OK) res = failed_result();
         }
         rhpdhg_batch_remove(s->batch, r.slot);
         r.slot = -1;
@@ -222,7 +230,9 @@ void worker_loop(rhpdhg_server *s) {
         res.y = r.y.data();
         res.cert_x = r.cx.data();
         res.cert_y = r.cy.data();
-        if (rhpdhg_poll(r.h, &res) == RHPDHG_BUSY) continue;
+        const int rc = rhpdhg_poll(r.h, &res);
+        if (rc == RHPDHG_BUSY) continue;
+        if (rc != RHPDHG_OK) res = failed_result();
         rhpdhg_free(r.h);
         r.h = nullptr;
         s->in_use -= r.bytes;
