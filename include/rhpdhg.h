@@ -390,7 +390,10 @@ int rhpdhg_probe_l2_read_bandwidth(int64_t bytes, void *cuda_stream, double *gbs
 typedef struct rhpdhg_batch rhpdhg_batch;
 
 /* Creates a batch with max_slots slots and a device arena of arena_bytes for the LPs' data.
- * cuda_stream: stream of all work (NULL = a private stream). */
+ * cuda_stream: stream of all work (NULL = a private stream).  The arena and a table of max_slots
+ * entries are all the device memory a batch uses.  In host memory it keeps, until it is freed,
+ * staging for the arrays of the largest LP added and for the largest result polled into host
+ * memory, up to half as much again as they need (pinned where pinned memory can be had). */
 int rhpdhg_batch_create(int32_t max_slots, int64_t arena_bytes, void *cuda_stream,
                         rhpdhg_batch **out);
 
@@ -400,8 +403,11 @@ int rhpdhg_batch_create(int32_t max_slots, int64_t arena_bytes, void *cuda_strea
  * FP64 anchors, and its restarts, restart points and checks in FP64, like rhpdhg_solve (the
  * restart-norm sums are FP32 within each warp and FP64 across warps; a near-certificate at a
  * restart point moves the slot to FP64 for the rest of its solve).
+ * lp's arrays may be freed on return.  The copies to the device are ordered on the batch's stream
+ * and not waited for, so an error of theirs is reported by a later call on the batch.
  * Returns RHPDHG_BUSY when no slot is free and RHPDHG_ERR_OOM when the arena lacks
- * rhpdhg_batch_bytes_needed(lp, precision) contiguous bytes. */
+ * rhpdhg_batch_bytes_needed(lp, precision) contiguous bytes or the host has no memory for the
+ * staging. */
 int rhpdhg_batch_add(rhpdhg_batch *b, const rhpdhg_problem *lp, const rhpdhg_params *params,
                      int32_t *slot);
 
@@ -409,7 +415,8 @@ int rhpdhg_batch_add(rhpdhg_batch *b, const rhpdhg_problem *lp, const rhpdhg_par
  * then iterates).  Synchronises the batch stream and refreshes every slot's status. */
 int rhpdhg_batch_step(rhpdhg_batch *b, int32_t iters);
 
-/* RHPDHG_BUSY while the slot's LP runs; then fills *r like rhpdhg_poll (solve_seconds = 0). */
+/* RHPDHG_BUSY while the slot's LP runs; then fills *r like rhpdhg_poll (solve_seconds = 0).  After an
+ * error nothing but the caller's vectors has been written; the slot keeps its result. */
 int rhpdhg_batch_poll(rhpdhg_batch *b, int32_t slot, rhpdhg_result *r);
 
 /* Frees a slot (finished or not) and its arena region. */

@@ -14,12 +14,12 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <string>
 #include <vector>
 
 #include "../../include/rhpdhg.h"
-#include "bufcache.h"
 #include "internal.h"
 #include "iter_common.cuh"
 #include "iter_mx_common.cuh"
@@ -663,25 +663,27 @@ k_batch(const BatchDesc *__restrict__ descs, int nslots, int iters) {
   if (threadIdx.x == 0) *home = ctls;
 }
 
-// What a poll gives back of a slot, in one array: x = E x~ of the last check (n), y = D y~ (m),
-// where a slot still in mixed precision holds y~ as y0 + dyt, the certificate's parts (n, m) and
-// sigma_max.
+// What a poll gives back of a slot: x = E x~ of the last check (n), y = D y~ (m), where a slot still
+// in mixed precision holds y~ as y0 + dyt, the certificate's parts (n, m) and sigma_max.  All of it in
+// one array in pinned memory (out), or x and y in the slot's scratch, which nothing uses between
+// steps (out NULL): either way a poll needs no device memory outside the arena.
 __global__ void k_batch_result(const BatchDesc *__restrict__ descs, int slot, int moved,
                                double *out) {
   const BatchDesc &d = descs[slot];
   const bool mixed = d.mixed && d.ic->mixed;
   const double *cx = moved ? d.cv_.certx2 : d.cv_.certx, *cy = moved ? d.rv_.certy2 : d.rv_.certy;
-  double *yo = out + d.n, *cxo = yo + d.m, *cyo = cxo + d.n;
+  double *xo = out ? out : d.tmp_n, *yo = out ? out + d.n : d.tmp_m;
+  double *cxo = out + d.n + d.m, *cyo = cxo + d.n;
   const int at = threadIdx.x + blockIdx.x * blockDim.x, step = blockDim.x * gridDim.x;
   for (int j = at; j < d.n; j += step) {
-    out[j] = d.cv_.e[j] * d.cv_.xout[j];
-    cxo[j] = cx[j];
+    xo[j] = d.cv_.e[j] * d.cv_.xout[j];
+    if (out) cxo[j] = cx[j];
   }
   for (int i = at; i < d.m; i += step) {
     yo[i] = d.rv_.d[i] * (mixed ? d.rvm.y0[i] + (double)d.rvm.dyt[i] : d.rv_.yt[i]);
-    cyo[i] = cy[i];
+    if (out) cyo[i] = cy[i];
   }
-  if (at == 0) cyo[d.m] = d.setup_out[0];
+  if (out && at == 0) cyo[d.m] = d.setup_out[0];
 }
 
 int pick_group(double avg) {
@@ -707,6 +709,11 @@ struct rhpdhg_batch {
   char *arena = nullptr;
   size_t arena_bytes = 0;
   struct Region { size_t off, size; };
+  struct HostBuf {                         // host memory for transfers: pinned where it can be had
+    char *p = nullptr;
+    size_t bytes = 0;
+    bool pinned = false;
+  };
   std::vector<Region> free_list;           // sorted by offset
   std::vector<Region> slot_region;
   std::vector<rh::BatchDesc> host_desc;
@@ -716,11 +723,9 @@ struct rhpdhg_batch {
   rh::BatchDesc *d_desc = nullptr;
   rh::Ctl *d_ctls = nullptr;               // every slot's control block (contiguous)
   rh::Ctl *h_ctl = nullptr;                // pinned copies of them
-  // pinned staging of an added LP's arrays (one copy to the arena instead of nine from pageable
-  // memory), free again when `staged` has passed; device and pinned copies of a polled result
-  char *h_stage = nullptr, *h_out = nullptr;
-  double *d_out = nullptr;
-  size_t stage_bytes = 0, out_bytes = 0;
+  // staging of an added LP's arrays (one copy to the arena instead of nine), free again when
+  // `staged` has passed; a polled result as the device writes it
+  HostBuf stage, out;
   cudaEvent_t staged = nullptr;
   cudaGraphExec_t gexec = nullptr;
   int graph_iters = -1;
@@ -779,34 +784,33 @@ void arena_release(rhpdhg_batch *b, size_t off, size_t size) {
   }
 }
 
-// Grows the pinned staging area to at least `bytes`, once nothing in flight reads it.
-cudaError_t stage_reserve(rhpdhg_batch *b, size_t bytes) {
-  cudaError_t e = cudaEventSynchronize(b->staged);
-  if (e != cudaSuccess || bytes <= b->stage_bytes) return e;
-  cudaFreeHost(b->h_stage);
-  b->h_stage = nullptr;
-  b->stage_bytes = 0;
-  bytes += bytes / 2;
-  e = cudaHostAlloc((void **)&b->h_stage, bytes, cudaHostAllocDefault);
-  if (e == cudaSuccess) b->stage_bytes = bytes;
-  return e;
+void host_release(rhpdhg_batch::HostBuf *h) {
+  if (h->pinned) cudaFreeHost(h->p);
+  else std::free(h->p);
+  *h = rhpdhg_batch::HostBuf();
 }
 
-// Grows the two copies of a polled result (the stream is idle: every poll ends with a
-// synchronisation).
-cudaError_t out_reserve(rhpdhg_batch *b, size_t bytes) {
-  if (bytes <= b->out_bytes) return cudaSuccess;
-  rh::buf_release(b->d_out);
-  cudaFreeHost(b->h_out);
-  b->d_out = nullptr;
-  b->h_out = nullptr;
-  b->out_bytes = 0;
-  bytes += bytes / 2;
-  cudaError_t e = rh::buf_alloc((void **)&b->d_out, bytes);
-  if (e == cudaSuccess) e = cudaHostAlloc((void **)&b->h_out, bytes, cudaHostAllocDefault);
-  if (e == cudaSuccess) b->out_bytes = bytes;
-  return e;
+// Grows h to at least `bytes` (nothing in flight uses it): pinned memory, and half as much again for
+// the next LP; else, if pageable memory will do, that.  False: none was to be had.
+bool host_reserve(rhpdhg_batch::HostBuf *h, size_t bytes, bool pageable) {
+  if (bytes <= h->bytes) return true;
+  host_release(h);
+  for (const size_t want : {bytes + bytes / 2, bytes}) {
+    if (cudaHostAlloc((void **)&h->p, want, cudaHostAllocMapped) == cudaSuccess) {
+      h->bytes = want;
+      h->pinned = true;
+      return true;
+    }
+    cudaGetLastError();
+    h->p = nullptr;
+  }
+  if (!pageable) return false;
+  h->p = (char *)std::malloc(bytes);
+  if (h->p) h->bytes = bytes;
+  return h->p != nullptr;
 }
+
+int result_blocks(const rh::BatchDesc &d) { return std::min(64, (std::max(d.n, d.m) + 255) / 256); }
 
 int berr(rhpdhg_batch *b, int code, const std::string &msg) {
   if (b) b->err = msg;
@@ -1001,17 +1005,17 @@ int rhpdhg_batch_add(rhpdhg_batch *b, const rhpdhg_problem *lp, const rhpdhg_par
   ic0.trace = nullptr;
   ic0.mixed = mixed ? 1 : 0;
   ic0.no_upper = any_upper ? 0 : 1;
-  // staged in pinned memory at the arena's offsets, the control block and descriptor behind them
+  // staged at the arena's offsets, the control block and descriptor behind them
   cudaStream_t st = b->st;
   const size_t at_ctl = upload, at_desc = at_ctl + align256(sizeof(c0));
-  cudaError_t e = stage_reserve(b, at_desc + align256(sizeof(d)));
-  if (e != cudaSuccess) {
-    cudaGetLastError();
+  cudaError_t e = cudaEventSynchronize(b->staged);
+  if (e != cudaSuccess || !host_reserve(&b->stage, at_desc + align256(sizeof(d)), true)) {
     arena_release(b, off, need);
-    return berr(b, e == cudaErrorMemoryAllocation ? RHPDHG_ERR_OOM : RHPDHG_ERR_CUDA,
-                std::string("batch add: ") + cudaGetErrorString(e));
+    if (e == cudaSuccess) return berr(b, RHPDHG_ERR_OOM, "batch add: out of host memory");
+    return berr(b, RHPDHG_ERR_CUDA, std::string("batch add: ") + cudaGetErrorString(e));
   }
-  auto host = [&](const void *dev) { return b->h_stage + ((const char *)dev - base); };
+  char *const stage = b->stage.p;
+  auto host = [&](const void *dev) { return stage + ((const char *)dev - base); };
   int *rp32 = (int *)host(d_rp), *h_cp = (int *)host(d_cp), *h_ri = (int *)host(d_ri);
   double *h_cv = (double *)host(d_cv);
   for (int i = 0; i <= m; ++i) rp32[i] = (int)rp[i];
@@ -1031,14 +1035,14 @@ int rhpdhg_batch_add(rhpdhg_batch *b, const rhpdhg_problem *lp, const rhpdhg_par
   std::memcpy(host(u), lp->u, n * 8);
   if (m) std::memcpy(host(q), lp->rhs, m * 8);
   std::memcpy(host(ic), &ic0, sizeof(ic0));
-  std::memcpy(b->h_stage + at_ctl, &c0, sizeof(c0));
-  std::memcpy(b->h_stage + at_desc, &d, sizeof(d));
-  e = cudaMemcpyAsync(base, b->h_stage, upload, cudaMemcpyHostToDevice, st);
+  std::memcpy(stage + at_ctl, &c0, sizeof(c0));
+  std::memcpy(stage + at_desc, &d, sizeof(d));
+  e = cudaMemcpyAsync(base, stage, upload, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(certx, 0, zeroed, st);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(ctl, b->h_stage + at_ctl, sizeof(c0), cudaMemcpyHostToDevice, st);
+    e = cudaMemcpyAsync(ctl, stage + at_ctl, sizeof(c0), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(b->d_desc + slot, b->h_stage + at_desc, sizeof(d), cudaMemcpyHostToDevice,
+    e = cudaMemcpyAsync(b->d_desc + slot, stage + at_desc, sizeof(d), cudaMemcpyHostToDevice,
                         st);
   if (e == cudaSuccess) e = cudaEventRecord(b->staged, st);
   if (e != cudaSuccess) {
@@ -1089,6 +1093,49 @@ int rhpdhg_batch_poll(rhpdhg_batch *b, int32_t slot, rhpdhg_result *r) {
   const rh::Ctl &c = b->h_ctl[slot];
   if (c.status == rh::kRunning) return RHPDHG_BUSY;
   const rh::BatchDesc &d = b->host_desc[slot];
+  const size_t m = d.m, n = d.n;
+  const bool mv = c.cert_src == rh::kCertAnchorMove;
+  const bool device = r->out_memory == RHPDHG_MEM_DEVICE;
+  // through pinned memory of the batch in one piece; without it, and to device memory, each vector
+  // from the arena (nothing of the result is filled before all of it has arrived)
+  const size_t count = 2 * (n + m) + 1;
+  double *got = nullptr;
+  cudaError_t e = cudaSuccess;
+  if (!device && host_reserve(&b->out, count * sizeof(double), false)) {
+    got = (double *)b->out.p;
+    void *mapped = nullptr;
+    e = cudaHostGetDevicePointer(&mapped, got, 0);
+    if (e != cudaSuccess) return berr(b, RHPDHG_ERR_CUDA, cudaGetErrorString(e));
+    e = rh::launch_kernel(rh::k_batch_result, result_blocks(d), 256, 0, b->st, b->d_desc, slot,
+                          mv ? 1 : 0, (double *)mapped);
+  } else {
+    e = rh::launch_kernel(rh::k_batch_result, result_blocks(d), 256, 0, b->st, b->d_desc, slot,
+                          mv ? 1 : 0, (double *)nullptr);
+  }
+  b->launches += 1;
+  // the four vectors: where the caller wants them, and where they are in got and in the arena
+  const struct { double *to; size_t at, len; const double *from; } parts[4] = {
+      {r->x, 0, n, d.tmp_n},
+      {r->y, n, m, d.tmp_m},
+      {r->cert_x, n + m, n, mv ? d.cv_.certx2 : d.cv_.certx},
+      {r->cert_y, 2 * n + m, m, mv ? d.rv_.certy2 : d.rv_.certy}};
+  double sigma = 0.0;
+  if (!got) {
+    const cudaMemcpyKind kind = device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+    for (const auto &p : parts)
+      if (e == cudaSuccess && p.to && p.len)
+        e = cudaMemcpyAsync(p.to, p.from, p.len * 8, kind, b->st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(&sigma, d.setup_out, 8, cudaMemcpyDeviceToHost, b->st);
+  }
+  const cudaError_t es = cudaStreamSynchronize(b->st);
+  if (e == cudaSuccess) e = es;
+  if (e != cudaSuccess) return berr(b, RHPDHG_ERR_CUDA, cudaGetErrorString(e));
+  if (got) {
+    for (const auto &p : parts)
+      if (p.to && p.len) std::memcpy(p.to, got + p.at, p.len * 8);
+    sigma = got[count - 1];
+  }
   r->status = c.status;
   r->iters = c.t;
   r->restarts = c.n;
@@ -1101,39 +1148,8 @@ int rhpdhg_batch_poll(rhpdhg_batch *b, int32_t slot, rhpdhg_result *r) {
   r->solve_seconds = 0.0;
   r->eta = c.eta;
   r->omega = c.omega;
-  const int m = d.m, n = d.n;
-  const bool mv = c.cert_src == rh::kCertAnchorMove;
+  r->sigma_max = sigma;
   r->cert_source = c.cert_src;
-  const size_t count = 2 * ((size_t)n + m) + 1;
-  cudaError_t e = out_reserve(b, count * sizeof(double));
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return berr(b, e == cudaErrorMemoryAllocation ? RHPDHG_ERR_OOM : RHPDHG_ERR_CUDA,
-                std::string("batch poll: ") + cudaGetErrorString(e));
-  }
-  const int blocks = std::min(64, (std::max(n, m) + 255) / 256);
-  rh::k_batch_result<<<blocks, 256, 0, b->st>>>(b->d_desc, slot, mv ? 1 : 0, b->d_out);
-  b->launches += 1;
-  // the four vectors' places in the result and in the caller's buffers
-  const struct { double *to; size_t at, len; } parts[4] = {
-      {r->x, 0, (size_t)n}, {r->y, (size_t)n, (size_t)m},
-      {r->cert_x, (size_t)n + m, (size_t)n}, {r->cert_y, 2 * (size_t)n + m, (size_t)m}};
-  const bool device = r->out_memory == RHPDHG_MEM_DEVICE;
-  if (device) {
-    for (const auto &p : parts)
-      if (p.to && p.len)
-        cudaMemcpyAsync(p.to, b->d_out + p.at, p.len * 8, cudaMemcpyDeviceToDevice, b->st);
-    cudaMemcpyAsync(b->h_out, b->d_out + count - 1, 8, cudaMemcpyDeviceToHost, b->st);
-  } else {
-    cudaMemcpyAsync(b->h_out, b->d_out, count * 8, cudaMemcpyDeviceToHost, b->st);
-  }
-  e = cudaStreamSynchronize(b->st);
-  if (e != cudaSuccess) return berr(b, RHPDHG_ERR_CUDA, cudaGetErrorString(e));
-  const double *got = (const double *)b->h_out;
-  r->sigma_max = device ? got[0] : got[count - 1];
-  if (!device)
-    for (const auto &p : parts)
-      if (p.to && p.len) std::memcpy(p.to, got + p.at, p.len * 8);
   return RHPDHG_OK;
 }
 
@@ -1175,9 +1191,8 @@ void rhpdhg_batch_free(rhpdhg_batch *b) {
   if (b->st) cudaStreamSynchronize(b->st);
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
   if (b->staged) cudaEventDestroy(b->staged);
-  if (b->h_stage) cudaFreeHost(b->h_stage);
-  if (b->h_out) cudaFreeHost(b->h_out);
-  rh::buf_release(b->d_out);
+  host_release(&b->stage);
+  host_release(&b->out);
   cudaFree(b->arena);
   cudaFree(b->d_desc);
   cudaFree(b->d_ctls);
