@@ -959,8 +959,8 @@ int rhpdhg_create(const rhpdhg_problem *lp, const rhpdhg_params *params, void *c
       CKT(cudaMemcpy(hcp.data(), cp, (n + 1) * sizeof(int), cudaMemcpyDeviceToHost));
       h->tune_sig = shape_signature(h, hrp, hcp);
     }
-    CKT(build_side(st, m, nnz, rp, col, val, h->D, h->E, lowp, &h->rows));
-    CKT(build_side(st, n, nnz, cp, ridx, cval, h->E, h->D, lowp, &h->cols));
+    CKT(build_side(st, m, rp, col, val, h->D, h->E, lowp, &h->rows));
+    CKT(build_side(st, n, cp, ridx, cval, h->E, h->D, lowp, &h->cols));
   }
   // ---- scaled vectors ----
   CKT(dalloc(&h->c, n));

@@ -119,7 +119,7 @@ void compute_scaling(cudaStream_t st, int m, int n, long long nnz, const int *rp
 // val * rscale[row] * cscale[col] (FP64, plus an FP32 copy for lowp 1 or a BF16 copy for lowp 2).
 // Rows longer than kShortMax, and the longest rows of any tile whose short segment would exceed
 // kSegBudget, go to the long CSR.  Device buffers come from buf_alloc.
-cudaError_t build_side(cudaStream_t st, int nrows, int nnz, const int *ptr, const int *idx,
+cudaError_t build_side(cudaStream_t st, int nrows, const int *ptr, const int *idx,
                        const double *val, const double *rscale, const double *cscale,
                        int lowp, SideStore *out);
 // Each entry of v (n positive factors) rounded to the nearest power of two on a log scale.

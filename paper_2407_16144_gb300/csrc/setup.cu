@@ -175,36 +175,66 @@ k_side_scale(int nrows, const int *__restrict__ ptr, const int *__restrict__ idx
   }
 }
 
-// copy each row's entries, scaled, to its place in the short or long arrays (G lanes per row: a
-// warp per row left most lanes idle on rows of a few entries), with an FP32
-// (LOWP 1) or BF16 (LOWP 2) copy of the scaled values
+// One scaled entry to its place in the short or long arrays, with an FP32 (LOWP 1) or BF16 (LOWP 2)
+// copy of the value.
+template <int LOWP>
+struct EntryOut {
+  int *idx;
+  double *val;
+  float *val32;
+  __nv_bfloat16 *val16;
+  __device__ __forceinline__ void put(int o, int j, double v) const {
+    idx[o] = j;
+    val[o] = v;
+    if (LOWP == 1) val32[o] = (float)v;
+    if (LOWP == 2) val16[o] = __float2bfloat16_rn((float)v);
+  }
+};
+
+// The short rows' entries, G lanes per row (a warp per row left most lanes idle on rows of a few
+// entries).
 template <int LOWP, int G>
 __global__ void __launch_bounds__(256)
 k_copy_rows(int nrows, const int *__restrict__ ptr, const int *__restrict__ idx,
             const double *__restrict__ val, const double *__restrict__ rs,
-            const double *__restrict__ cs, const int *__restrict__ dst,
-            const uint32_t *__restrict__ long_mask, int *idx_s, double *val_s, float *val32_s,
-            __nv_bfloat16 *val16_s, int *idx_l, double *val_l, float *val32_l,
-            __nv_bfloat16 *val16_l) {
+            const double *__restrict__ cs, const int *__restrict__ ptr_s,
+            const uint32_t *__restrict__ long_mask, EntryOut<LOWP> out) {
   const long long w = (blockIdx.x * 256LL + threadIdx.x) / G;
-  const int lane = threadIdx.x % G;
   if (w >= nrows) return;
   const int r = (int)w;
-  const bool lg = (long_mask[r >> 5] >> (r & 31)) & 1u;
-  int *ix = lg ? idx_l : idx_s;
-  double *vx = lg ? val_l : val_s;
-  float *vf = lg ? val32_l : val32_s;
-  __nv_bfloat16 *vh = lg ? val16_l : val16_s;
-  const int b = ptr[r], e = ptr[r + 1], o = dst[r];
+  if ((long_mask[r >> 5] >> (r & 31)) & 1u) return;
+  const int b = ptr[r], len = ptr[r + 1] - b, o = ptr_s[r];
   const double sr = rs[r];
 #pragma unroll 4
-  for (int p = b + lane; p < e; p += G) {
-    const int j = idx[p];
-    const double v = sr * val[p] * cs[j];
-    ix[o + (p - b)] = j;
-    vx[o + (p - b)] = v;
-    if (LOWP == 1) vf[o + (p - b)] = (float)v;
-    if (LOWP == 2) vh[o + (p - b)] = __float2bfloat16_rn((float)v);
+  for (int t = threadIdx.x % G; t < len; t += G) {
+    const int j = idx[b + t];
+    out.put(o + t, j, sr * val[b + t] * cs[j]);
+  }
+}
+
+// The long rows' entries, a warp per chunk with its eight entries a lane in flight.  (With the lanes
+// of a short row, chosen from the mean length, one row's dependent loads were the whole pass: in mixed
+// precision a row of 1M entries took 75.8 ms, with one warp 23.8, now 0.05; the power-law columns of
+// 2.5M entries 427 us, 182, now 63 with their short columns.)
+template <int LOWP>
+__global__ void __launch_bounds__(256)
+k_copy_chunks(int nchunks, const int4 *__restrict__ desc, const int *__restrict__ long_rows,
+              const int *__restrict__ beg_l, const int *__restrict__ ptr,
+              const int *__restrict__ idx, const double *__restrict__ val,
+              const double *__restrict__ rs, const double *__restrict__ cs, EntryOut<LOWP> out) {
+  const long long w = (blockIdx.x * 256LL + threadIdx.x) / kWarp;
+  if (w >= nchunks) return;
+  const int4 d = desc[w];                      // long row, entries [d.y, d.z) of the long array
+  const int r = long_rows[d.x], len = d.z - d.y;
+  const int b = ptr[r] + (d.y - beg_l[d.x]);
+  const double sr = rs[r];
+#pragma unroll
+  for (int u = 0; u < kChunk / kWarp; ++u) {
+    const int t = u * kWarp + threadIdx.x % kWarp;
+    if (t < len) {
+      const int j = idx[b + t];
+      out.put(d.y + t, j, sr * val[b + t] * cs[j]);
+    }
   }
 }
 
@@ -510,7 +540,7 @@ k_plan_scan(int nblocks, PlanBlock *blocks, PlanBlock *all) {
 
 __global__ void __launch_bounds__(kPlanThreads)
 k_plan_emit(int nrows, int ntiles, const int *__restrict__ ptr, const PlanTile *tiles,
-            const PlanBlock *blocks, int *ptr_s, int *tile_end, int *dst, uint32_t *long_mask,
+            const PlanBlock *blocks, int *ptr_s, int *tile_end, uint32_t *long_mask,
             int *long_rows, int *beg_l, int *end_l, int *chunk_ptr, int *chunk_row) {
   __shared__ PlanCount sh[kPlanTiles];      // what precedes each tile, from the block's start
   const unsigned full = 0xffffffffu;
@@ -552,7 +582,6 @@ k_plan_emit(int nrows, int ntiles, const int *__restrict__ ptr, const PlanTile *
       if (lane >= o) incl += v;
     }
     const int start = (int)at.s + incl - (lg ? 0 : len);
-    int to = start;
     if (mask) {                              // warp-uniform
       const int nc = lg ? (len + kChunk - 1) / kChunk : 0;
       const long long pl = lg ? ((long long)len + 3) & ~3LL : 0;
@@ -568,7 +597,7 @@ k_plan_emit(int nrows, int ntiles, const int *__restrict__ ptr, const PlanTile *
       }
       const int row = at.nl + __popc(mask & ((1u << lane) - 1u));
       if (lg) {
-        to = (int)(at.l + li - pl);
+        const int to = (int)(at.l + li - pl);
         long_rows[row] = (int)r;
         beg_l[row] = to;
         end_l[row] = to + len;
@@ -581,10 +610,7 @@ k_plan_emit(int nrows, int ntiles, const int *__restrict__ ptr, const PlanTile *
         for (int c = c1 - n + lane; c < c1; c += 32) chunk_row[c] = id;
       }
     }
-    if (r < nrows) {
-      ptr_s[r] = start;
-      dst[r] = to;
-    }
+    if (r < nrows) ptr_s[r] = start;
     if (lane == 0) {
       tile_end[t] = (int)at.s + tiles[t].seg;
       long_mask[t] = mask;
@@ -1007,14 +1033,13 @@ bool plan_side(const int *hp, int nrows, SidePlan *p) {
   return true;
 }
 
-cudaError_t build_side(cudaStream_t st, int nrows, int nnz, const int *ptr, const int *idx,
+cudaError_t build_side(cudaStream_t st, int nrows, const int *ptr, const int *idx,
                        const double *val, const double *rscale, const double *cscale,
                        int lowp, SideStore *out) {
   SideStore s;
   cudaError_t err = cudaSuccess;
   const int ntiles = (int)(((long long)nrows + kTileRows - 1) / kTileRows);
   const int nplan = (ntiles + kPlanTiles - 1) / kPlanTiles;
-  int *d_dst = nullptr;
   PlanTile *d_tiles = nullptr;
   PlanBlock *d_blocks = nullptr;
   PlanBlock tot{};
@@ -1075,11 +1100,10 @@ cudaError_t build_side(cudaStream_t st, int nrows, int nnz, const int *ptr, cons
   TRY(get(&s.chunk_ptr, (size_t)nlong + 1));
   TRY(get(&s.chunk_row, nch));
   TRY(get(&s.chunk_desc, nch));
-  TRY(get(&d_dst, nrows));
   TRY(get(&s.long_mask, ntiles));
   if (ntiles > 0) {
     k_plan_emit<<<nplan, kPlanThreads, 0, st>>>(nrows, ntiles, ptr, d_tiles, d_blocks, s.ptr_s,
-                                                s.tile_end, d_dst, s.long_mask, s.long_rows,
+                                                s.tile_end, s.long_mask, s.long_rows,
                                                 s.beg_l, s.end_l, s.chunk_ptr, s.chunk_row);
     count_launches(1);
     if (nch > 0) {
@@ -1109,17 +1133,22 @@ cudaError_t build_side(cudaStream_t st, int nrows, int nnz, const int *ptr, cons
     TRY(cudaMemsetAsync(s.val16_l, 0, nnz_l * sizeof(__nv_bfloat16), st));
   }
   if (nrows > 0) {
-    with_group<4>(nnz, nrows, [&](auto G) {
-      auto copy = [&](auto kern) {
-        kern<<<nblocks((long long)nrows * G(), 256), 256, 0, st>>>(
-            nrows, ptr, idx, val, rscale, cscale, d_dst, s.long_mask, s.idx_s, s.val64_s,
-            s.val32_s, s.val16_s, s.idx_l, s.val64_l, s.val32_l, s.val16_l);
-      };
-      if (lowp == 1) copy(k_copy_rows<1, G()>);
-      else if (lowp == 2) copy(k_copy_rows<2, G()>);
-      else copy(k_copy_rows<0, G()>);
-    });
-    count_launches(1);
+    auto copy = [&](auto LP) {
+      const EntryOut<LP()> shorts{s.idx_s, s.val64_s, s.val32_s, s.val16_s};
+      const EntryOut<LP()> longs{s.idx_l, s.val64_l, s.val32_l, s.val16_l};
+      with_group<4>(tot.c.s, nrows, [&](auto G) {
+        k_copy_rows<LP(), G()><<<nblocks((long long)nrows * G(), 256), 256, 0, st>>>(
+            nrows, ptr, idx, val, rscale, cscale, s.ptr_s, s.long_mask, shorts);
+      });
+      count_launches(1);
+      if (nch == 0) return;
+      k_copy_chunks<LP()><<<nblocks((long long)nch * kWarp, 256), 256, 0, st>>>(
+          nch, s.chunk_desc, s.long_rows, s.beg_l, ptr, idx, val, rscale, cscale, longs);
+      count_launches(1);
+    };
+    if (lowp == 1) copy(std::integral_constant<int, 1>{});
+    else if (lowp == 2) copy(std::integral_constant<int, 2>{});
+    else copy(std::integral_constant<int, 0>{});
   }
   // ---- walk scratch ------------------------------------------------------------------------
   TRY(buf_alloc((void **)&s.part_a, (size_t)std::max(nch, 1) * sizeof(double)));
@@ -1133,7 +1162,6 @@ cudaError_t build_side(cudaStream_t st, int nrows, int nnz, const int *ptr, cons
   TRY(cudaStreamSynchronize(st));
   TRY(cudaGetLastError());
 #undef TRY
-  buf_release(d_dst);
   buf_release(d_tiles);
   buf_release(d_blocks);
   s.lay.ptr_s = s.ptr_s;
@@ -1163,7 +1191,6 @@ cudaError_t build_side(cudaStream_t st, int nrows, int nnz, const int *ptr, cons
   return cudaSuccess;
 fail:
   cudaStreamSynchronize(st);
-  buf_release(d_dst);
   buf_release(d_tiles);
   buf_release(d_blocks);
   free_side(&s);
