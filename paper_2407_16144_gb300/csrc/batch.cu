@@ -130,7 +130,8 @@ __device__ __forceinline__ void rows_apply(int nrows, const int *ptr, const int 
     const int rb = ptr[min(row, nrows)], re = ptr[min(row + 1, nrows)];
     VT mine = VT(0);
     for (int pass0 = 0; pass0 < g; pass0 += kRowPasses) {
-      int p0[kRowPasses], pe[kRowPasses], j[kRowPasses][kRowSteps];
+      unsigned p0[kRowPasses], pe[kRowPasses];     // (unsigned: see for_strided)
+      int j[kRowPasses][kRowSteps];
       VT v[kRowPasses][kRowSteps], x[kRowPasses][kRowSteps], s[kRowPasses];
 #pragma unroll
       for (int u = 0; u < kRowPasses; ++u) {
@@ -143,7 +144,7 @@ __device__ __forceinline__ void rows_apply(int nrows, const int *ptr, const int 
       for (int u = 0; u < kRowPasses; ++u)
 #pragma unroll
         for (int t = 0; t < kRowSteps; ++t) {
-          const int p = p0[u] + t * g;
+          const unsigned p = p0[u] + t * g;
           const bool in = p < pe[u];
           j[u][t] = in ? idx[p] : 0;
           v[u][t] = in ? val[p] : VT(0);
@@ -159,7 +160,7 @@ __device__ __forceinline__ void rows_apply(int nrows, const int *ptr, const int 
 #pragma unroll
         for (int t = 0; t < kRowSteps; ++t)
           if (p0[u] + t * g < pe[u]) s[u] += v[u][t] * x[u][t];
-        for (int p = p0[u] + kRowSteps * g; p < pe[u]; p += g) s[u] += val[p] * VT(src(idx[p]));
+        for (unsigned p = p0[u] + kRowSteps * g; p < pe[u]; p += g) s[u] += val[p] * VT(src(idx[p]));
       }
       const int mypass = lane / rpp - pass0;        // the pass that sums this lane's own row
       if (g >= 4) {
@@ -197,7 +198,7 @@ __device__ void rows_stat(int nrows, const int *ptr, const int *idx, const doubl
     double s = 0.0;
     if (r < nrows) {
       const double sr = rs[r];
-      for (int p = ptr[r] + gl; p < ptr[r + 1]; p += g) {
+      for (unsigned p = ptr[r] + gl; p < (unsigned)ptr[r + 1]; p += g) {
         // (not fused with the sum, whatever the context compiles to: the factors' last bits reach a
         // mixed slot's FP32 values)
         const double a = __dmul_rn(__dmul_rn(fabs(val[p]), sr), cs[idx[p]]);

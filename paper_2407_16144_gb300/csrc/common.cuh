@@ -231,6 +231,14 @@ __device__ __forceinline__ double warp_max(double v) {
   return v;
 }
 
+// f(p) for p = b + first, b + first + step, ... below e.  Entry positions go up to the int32 limit, so
+// the step past the last one has to be taken in unsigned arithmetic.
+template <class F>
+__host__ __device__ __forceinline__ void for_strided(int b, int e, int first, int step, F f) {
+#pragma unroll 4
+  for (unsigned p = (unsigned)b + (unsigned)first; p < (unsigned)e; p += (unsigned)step) f((int)p);
+}
+
 // ---------------------------------------------------------------------------------------------
 // FP64 comparisons on the integer pipe.  The FP64 pipe of this part takes about 19 clocks per warp
 // and SM for any instruction, a comparison, a maximum or an isfinite as long as a fused

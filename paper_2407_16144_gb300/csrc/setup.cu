@@ -140,10 +140,8 @@ k_side_scale(int nrows, const int *__restrict__ ptr, const int *__restrict__ idx
   // (a sum keeps one order, that of its G lanes: its last bits reach mixed-precision results)
   const bool lg = OP == 0 && pe - pb > kStatLong * G;
   StatAcc<OP> acc;
-  if (!lg) {
-#pragma unroll 4
-    for (int p = pb + sub; p < pe; p += G) acc.add(fabs(val[p]), sr, cs[idx[p]], alpha);
-  }
+  if (!lg)
+    for_strided(pb, pe, sub, G, [&](int p) { acc.add(fabs(val[p]), sr, cs[idx[p]], alpha); });
 #pragma unroll
   for (int o = G / 2; o > 0; o >>= 1) acc.join(__shfl_xor_sync(0xffffffffu, acc.s, o, G));
   if (sub == 0) {
@@ -156,8 +154,8 @@ k_side_scale(int nrows, const int *__restrict__ ptr, const int *__restrict__ idx
     const double sq = rs[q];
     const int qe = ptr[q + 1];
     StatAcc<OP> a;
-#pragma unroll 4
-    for (int p = ptr[q] + threadIdx.x; p < qe; p += 256) a.add(fabs(val[p]), sq, cs[idx[p]], alpha);
+    for_strided(ptr[q], qe, threadIdx.x, 256,
+                [&](int p) { a.add(fabs(val[p]), sq, cs[idx[p]], alpha); });
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) a.join(__shfl_xor_sync(0xffffffffu, a.s, o));
     if (threadIdx.x % 32 == 0) part[threadIdx.x / 32] = a.s;
