@@ -1,9 +1,10 @@
 // Device buffers of handles: allocated from, and returned to, a process-wide cache of freed
 // buffers (reuse of an exact size on the same device; at most kBufferCacheBytes held, the longest
-// unused given back first; the cache is dropped and the allocation retried when the device runs out of memory).  A buffer may be released only when
-// no work on it is pending (the stream that used it has been synchronised).  Creating and
-// freeing handles of the same sizes (a benchmark loop, a serving stream) then costs no device
-// allocation and no device-wide synchronisation after the first time.
+// unused given back first; the cache is dropped and the allocation retried when the device runs out
+// of memory).  A buffer may be released only when no work on it is pending (the stream that used it
+// has been synchronised).  Creating and freeing handles of the same sizes (a benchmark loop, a
+// serving stream) then costs no device allocation and no device-wide synchronisation after the first
+// time.
 #pragma once
 
 #include <cstddef>

@@ -6,10 +6,7 @@
 #include <algorithm>
 #include <atomic>
 #include <climits>
-#include <map>
-#include <mutex>
 #include <type_traits>
-#include <unordered_map>
 #include <utility>
 #include <vector>
 
@@ -764,147 +761,6 @@ void compute_scaling(cudaStream_t st, int m, int n, long long nnz, const int *rp
     std::swap(D, tmp_m);
     std::swap(E, tmp_n);
   }
-}
-
-namespace {
-// Cached buffers are keyed by (device, size): a buffer is only ever reused on the device it was
-// allocated on.  Buffers from a caller's allocator carry it (hook.free set) and are never cached.
-struct BufInfo {
-  int dev;
-  size_t bytes;
-  DevAllocator hook;
-};
-
-thread_local const DevAllocator *tl_alloc = nullptr;   // set by AllocScope
-std::mutex g_buf_mu;
-std::unordered_map<void *, BufInfo> g_buf_info;              // every buffer from buf_alloc
-// cached, by (device, size): the pointer and the release that brought it, oldest first
-std::map<std::pair<int, size_t>, std::vector<std::pair<void *, unsigned long long>>> g_buf_free;
-size_t g_buf_free_bytes = 0;
-unsigned long long g_buf_releases = 0;
-
-// Frees every cached buffer (on its own device); the caller holds g_buf_mu.
-void buf_drop_cache_locked() {
-  if (g_buf_free.empty()) return;
-  int cur = -1;
-  cudaGetDevice(&cur);
-  for (auto &kv : g_buf_free) {
-    if (kv.second.empty()) continue;
-    cudaSetDevice(kv.first.first);
-    for (const auto &b : kv.second) {
-      g_buf_info.erase(b.first);
-      cudaFree(b.first);
-    }
-  }
-  if (cur >= 0) cudaSetDevice(cur);
-  g_buf_free.clear();
-  g_buf_free_bytes = 0;
-}
-
-// Frees the cached buffers that were released longest ago until `bytes` more fit; the caller holds
-// g_buf_mu.  (Refusing the newcomer instead made every call that followed a larger handle allocate
-// and free its scratch again: a KKT evaluation of a 30M-entry LP 640 us instead of 464.)
-void buf_make_room_locked(size_t bytes) {
-  int cur = -1;
-  cudaGetDevice(&cur);
-  while (g_buf_free_bytes + bytes > kBufferCacheBytes) {
-    auto old = g_buf_free.end();
-    for (auto it = g_buf_free.begin(); it != g_buf_free.end(); ++it)
-      if (!it->second.empty() &&
-          (old == g_buf_free.end() || it->second.front().second < old->second.front().second))
-        old = it;
-    if (old == g_buf_free.end()) break;
-    void *p = old->second.front().first;
-    g_buf_free_bytes -= old->first.second;
-    cudaSetDevice(old->first.first);
-    g_buf_info.erase(p);
-    cudaFree(p);
-    old->second.erase(old->second.begin());
-    if (old->second.empty()) g_buf_free.erase(old);
-  }
-  if (cur >= 0) cudaSetDevice(cur);
-}
-}  // namespace
-
-AllocScope::AllocScope(const DevAllocator &a) : prev_(tl_alloc), mine_(a) {
-  tl_alloc = (mine_.alloc && mine_.free) ? &mine_ : nullptr;
-}
-AllocScope::~AllocScope() { tl_alloc = prev_; }
-
-cudaError_t buf_alloc(void **p, size_t bytes) {
-  bytes = std::max<size_t>(bytes, 1);
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (tl_alloc) {
-    // 256-byte alignment covers every vector load of the kernels
-    void *q = tl_alloc->alloc(bytes, tl_alloc->stream, tl_alloc->ctx);
-    if (!q) return cudaErrorMemoryAllocation;
-    if (reinterpret_cast<uintptr_t>(q) % 256 != 0) {
-      tl_alloc->free(q, tl_alloc->stream, tl_alloc->ctx);
-      return cudaErrorInvalidValue;
-    }
-    *p = q;
-    std::lock_guard<std::mutex> lk(g_buf_mu);
-    g_buf_info[q] = BufInfo{dev, bytes, *tl_alloc};
-    return cudaSuccess;
-  }
-  {
-    std::lock_guard<std::mutex> lk(g_buf_mu);
-    auto it = g_buf_free.find({dev, bytes});
-    if (it != g_buf_free.end() && !it->second.empty()) {
-      *p = it->second.back().first;
-      it->second.pop_back();
-      g_buf_free_bytes -= bytes;
-      return cudaSuccess;
-    }
-  }
-  e = cudaMalloc(p, bytes);
-  if (e == cudaErrorMemoryAllocation) {
-    cudaGetLastError();
-    {
-      std::lock_guard<std::mutex> lk(g_buf_mu);
-      buf_drop_cache_locked();
-    }
-    e = cudaMalloc(p, bytes);
-  }
-  if (e == cudaSuccess) {
-    std::lock_guard<std::mutex> lk(g_buf_mu);
-    g_buf_info[*p] = BufInfo{dev, bytes, DevAllocator()};
-  }
-  return e;
-}
-
-void buf_release(void *p) {
-  if (!p) return;
-  {
-    std::unique_lock<std::mutex> lk(g_buf_mu);
-    auto it = g_buf_info.find(p);
-    if (it != g_buf_info.end()) {
-      const BufInfo bi = it->second;
-      if (bi.hook.free) {
-        g_buf_info.erase(it);
-        lk.unlock();
-        bi.hook.free(p, bi.hook.stream, bi.hook.ctx);
-        return;
-      }
-      if (bi.bytes <= kBufferCacheBytes) {
-        if (g_buf_free_bytes + bi.bytes > kBufferCacheBytes) buf_make_room_locked(bi.bytes);
-        g_buf_free[{bi.dev, bi.bytes}].push_back({p, g_buf_releases++});
-        g_buf_free_bytes += bi.bytes;
-        return;
-      }
-      g_buf_info.erase(it);
-    }
-  }
-  cudaFree(p);
-}
-
-size_t buf_drop_cache() {
-  std::lock_guard<std::mutex> lk(g_buf_mu);
-  const size_t freed = g_buf_free_bytes;
-  buf_drop_cache_locked();
-  return freed;
 }
 
 // A side is skewed (its ordered FP64 tiles take tile_rows_wide) when summing its tiles' longest rows
