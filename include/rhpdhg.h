@@ -419,7 +419,7 @@ int rhpdhg_batch_step(rhpdhg_batch *b, int32_t iters);
  * error nothing but the caller's vectors has been written; the slot keeps its result. */
 int rhpdhg_batch_poll(rhpdhg_batch *b, int32_t slot, rhpdhg_result *r);
 
-/* Frees a slot (finished or not) and its arena region. */
+/* Frees a slot (finished or not) and its arena region; RHPDHG_ERR_CUDA: nothing was freed. */
 int rhpdhg_batch_remove(rhpdhg_batch *b, int32_t slot);
 
 /* Status of a slot after the last step (RHPDHG_STATUS_*), or -1 for an empty slot. */

@@ -1157,12 +1157,13 @@ int rhpdhg_batch_poll(rhpdhg_batch *b, int32_t slot, rhpdhg_result *r) {
 int rhpdhg_batch_remove(rhpdhg_batch *b, int32_t slot) {
   if (!b || slot < 0 || slot >= b->max_slots || !b->host_desc[slot].active)
     return RHPDHG_ERR_INVALID_ARG;
-  rh::BatchDesc d{};
-  d.active = 0;
-  cudaMemsetAsync(b->d_desc + slot, 0, sizeof(rh::BatchDesc), b->st);
-  cudaMemsetAsync(b->d_ctls + slot, 0, sizeof(rh::Ctl), b->st);
+  // (a slot that stayed in the device's table would go on iterating in memory given to another)
+  cudaError_t e = cudaMemsetAsync(b->d_desc + slot, 0, sizeof(rh::BatchDesc), b->st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_ctls + slot, 0, sizeof(rh::Ctl), b->st);
+  if (e != cudaSuccess)
+    return berr(b, RHPDHG_ERR_CUDA, std::string("batch remove: ") + cudaGetErrorString(e));
   arena_release(b, b->slot_region[slot].off, b->slot_region[slot].size);
-  b->host_desc[slot] = d;
+  b->host_desc[slot] = rh::BatchDesc{};
   b->slot_region[slot] = {0, 0};
   std::memset(&b->h_ctl[slot], 0, sizeof(rh::Ctl));
   return RHPDHG_OK;
