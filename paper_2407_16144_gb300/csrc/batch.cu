@@ -725,9 +725,9 @@ struct rhpdhg_batch {
   rh::Ctl *d_ctls = nullptr;               // every slot's control block (contiguous)
   rh::Ctl *h_ctl = nullptr;                // pinned copies of them
   // staging of an added LP's arrays (one copy to the arena instead of nine), free again when
-  // `staged` has passed; a polled result as the device writes it
+  // `pending` has passed; a polled result as the device writes it
   HostBuf stage, out;
-  cudaEvent_t staged = nullptr;
+  cudaEvent_t pending = nullptr;           // behind the last work that no call has waited for
   cudaGraphExec_t gexec = nullptr;
   int graph_iters = -1;
   std::string err;
@@ -842,7 +842,7 @@ int rhpdhg_batch_create(int32_t max_slots, int64_t arena_bytes, void *cuda_strea
   if (e == cudaSuccess) e = cudaMalloc(&b->d_desc, max_slots * sizeof(rh::BatchDesc));
   if (e == cudaSuccess) e = cudaMalloc(&b->d_ctls, max_slots * sizeof(rh::Ctl));
   if (e == cudaSuccess) e = cudaHostAlloc((void **)&b->h_ctl, max_slots * sizeof(rh::Ctl), 0);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->staged, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->pending, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     rhpdhg_batch_free(b);
     return berr(nullptr, RHPDHG_ERR_OOM, std::string("batch: ") + cudaGetErrorString(e));
@@ -1009,7 +1009,7 @@ int rhpdhg_batch_add(rhpdhg_batch *b, const rhpdhg_problem *lp, const rhpdhg_par
   // staged at the arena's offsets, the control block and descriptor behind them
   cudaStream_t st = b->st;
   const size_t at_ctl = upload, at_desc = at_ctl + align256(sizeof(c0));
-  cudaError_t e = cudaEventSynchronize(b->staged);
+  cudaError_t e = cudaEventSynchronize(b->pending);
   if (e != cudaSuccess || !host_reserve(&b->stage, at_desc + align256(sizeof(d)), true)) {
     arena_release(b, off, need);
     if (e == cudaSuccess) return berr(b, RHPDHG_ERR_OOM, "batch add: out of host memory");
@@ -1045,7 +1045,7 @@ int rhpdhg_batch_add(rhpdhg_batch *b, const rhpdhg_problem *lp, const rhpdhg_par
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(b->d_desc + slot, stage + at_desc, sizeof(d), cudaMemcpyHostToDevice,
                         st);
-  if (e == cudaSuccess) e = cudaEventRecord(b->staged, st);
+  if (e == cudaSuccess) e = cudaEventRecord(b->pending, st);
   if (e != cudaSuccess) {
     cudaStreamSynchronize(st);
     arena_release(b, off, need);
@@ -1163,6 +1163,7 @@ int rhpdhg_batch_remove(rhpdhg_batch *b, int32_t slot) {
   if (e != cudaSuccess)
     return berr(b, RHPDHG_ERR_CUDA, std::string("batch remove: ") + cudaGetErrorString(e));
   arena_release(b, b->slot_region[slot].off, b->slot_region[slot].size);
+  cudaEventRecord(b->pending, b->st);
   b->host_desc[slot] = rh::BatchDesc{};
   b->slot_region[slot] = {0, 0};
   std::memset(&b->h_ctl[slot], 0, sizeof(rh::Ctl));
@@ -1190,9 +1191,12 @@ int64_t rhpdhg_batch_launch_count(const rhpdhg_batch *b) { return b ? b->launche
 
 void rhpdhg_batch_free(rhpdhg_batch *b) {
   if (!b) return;
-  if (b->st) cudaStreamSynchronize(b->st);
+  // (the event, not the stream: a caller's stream may have been destroyed by now)
+  if (b->pending) {
+    cudaEventSynchronize(b->pending);
+    cudaEventDestroy(b->pending);
+  }
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
-  if (b->staged) cudaEventDestroy(b->staged);
   host_release(&b->stage);
   host_release(&b->out);
   cudaFree(b->arena);

@@ -1,6 +1,6 @@
-"""A batch on the caller's stream when calls on that stream fail: the failure is made on the host, by
-invalidating a stream capture, so that an asynchronous call on it returns an error and the device
-stays as it is."""
+"""A batch on the caller's stream: the stream destroyed before the batch, and calls that fail on it.
+The failure is made on the host, by invalidating a stream capture, so that an asynchronous call on the
+stream returns an error and the device stays as it is."""
 import ctypes as C
 
 import pytest
@@ -60,3 +60,21 @@ def test_remove_reports_a_slot_it_could_not_clear(rh, cudart):
         run(b, rh, slot)
         assert b.poll(slot).iters == 64
     assert cudart.cudaStreamDestroy(st) == 0
+
+
+@pytest.mark.parametrize("last", ["step", "remove", "add"])
+def test_batch_freed_after_its_stream(rh, cudart, last):
+    """Work that add and remove leave on the stream is waited for, without the stream itself."""
+    lp = lpgen.make_standard_planted(seed=3, m=60, n=150)
+    st = new_stream(cudart)
+    b = rh.Batch(2, 8 << 20, stream=st.value)
+    slot = b.add(lp, max_iters=64)
+    run(b, rh, slot)
+    if last != "step":
+        assert b.poll(slot).iters == 64
+    if last == "add":
+        b.add(lp, max_iters=64)
+    assert cudart.cudaStreamDestroy(st) == 0
+    b.close()
+    with rh.Solver(lp, max_iters=64) as s:                    # the device still answers
+        assert s.run().iters == 64
