@@ -300,11 +300,13 @@ int rhpdhg_get_trace(const rhpdhg_handle *h, rhpdhg_trace_rec *recs, int64_t cap
 #define RHPDHG_LAYOUT_FIELDS 19
 int rhpdhg_get_layout(const rhpdhg_handle *h, int64_t *out, int32_t capacity);
 
-/* Handles take their device buffers from a process-wide cache of buffers freed by earlier
- * handles (same device, same size; at most 4 GiB kept), so that creating and freeing handles of
- * the same sizes costs no device allocation after the first time.  This frees every cached
- * buffer (for instance before a device reset, or to give the memory back) and returns the bytes
- * freed.  Handles alive at the time are not affected. */
+/* Handles and rhpdhg_kkt_eval take their device buffers from a process-wide cache of buffers
+ * released earlier (same device, same size; at most 4 GiB kept, those released longest ago given
+ * back first), so that creating and freeing handles of the same sizes costs no device allocation
+ * after the first time.  Freed handles also leave their pinned copies of the control block for later
+ * ones (at most 64, of two control blocks each).  This frees every cached buffer and every such
+ * copy (for instance before a device reset, or to give the memory back) and returns the bytes of
+ * device memory freed.  Handles and batches alive at the time are not affected. */
 int64_t rhpdhg_release_cached_memory(void);
 
 /* Plan of the tiled split-CSR layout that rhpdhg_create builds for an operator side (K^ or K^T)
@@ -337,8 +339,9 @@ int rhpdhg_kernel_times(const rhpdhg_handle *h, double *ms_row, double *ms_col,
  * [0, nnz] or decrease, and an entry whose column leaves [0, n), are skipped on the device and
  * the call then returns RHPDHG_ERR_INVALID_ARG.  Work is ordered on `cuda_stream` (NULL = legacy
  * default stream) and the call synchronises it, so it must not be issued on a stream that is
- * being captured into a graph.  Scratch (n + 8200 doubles) is allocated with cudaMalloc and
- * freed before returning.  Errors: RHPDHG_ERR_INVALID_ARG for host-memory, incomplete or
+ * being captured into a graph.  Scratch (n + 8200 doubles of device memory) is taken from the
+ * process-wide cache of device buffers and goes back to it, so it stays allocated after the call
+ * until it is evicted or rhpdhg_release_cached_memory is called.  Errors: RHPDHG_ERR_INVALID_ARG for host-memory, incomplete or
  * out-of-range input, RHPDHG_ERR_OOM / RHPDHG_ERR_CUDA on CUDA failures; each sets the message
  * of rhpdhg_last_error(NULL). */
 int rhpdhg_kkt_eval(const rhpdhg_problem *lp, const double *x, const double *y,

@@ -76,3 +76,26 @@ def test_kkt_rows_match_numpy(name):
     assert rc == rh.OK, rh.rhpdhg_last_error(None)
     for a, b, t in zip(got, want, tol):
         assert abs(a - b) <= t, (got, want, tol)
+
+
+def test_kkt_scratch_stays_in_the_buffer_cache():
+    """n + 8200 doubles after the first call, no more after the second, given back on request."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2407_16144_gb300 import _build, rhpdhg as rh
+    _build.build()
+    rh.load()
+    n = 1000
+    f64 = dict(dtype=torch.float64, device="cuda")
+    lp = lpgen.LP(m_eq=1, m_ineq=0, n=n, row_ptr=torch.tensor([0, 1], device="cuda"),
+                  col_idx=torch.zeros(1, dtype=torch.int32, device="cuda"), val=torch.ones(1, **f64),
+                  c=torch.ones(n, **f64), q=torch.ones(1, **f64), l=torch.zeros(n, **f64),
+                  u=torch.ones(n, **f64))
+    x, y = torch.ones(n, **f64), torch.ones(1, **f64)
+    rh.release_cached_memory()
+    for _ in range(2):
+        rc, out = rh.rhpdhg_kkt_eval(rh.device_problem(lp), x.data_ptr(), y.data_ptr())
+        assert rc == rh.OK
+    assert rh.release_cached_memory() == 8 * (n + 8200)
+    assert rh.release_cached_memory() == 0
