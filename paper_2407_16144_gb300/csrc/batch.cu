@@ -30,8 +30,10 @@ namespace {
 
 // Threads per CTA of the batched kernel: 16 warps of at most 128 registers, a whole SM.  (8 warps of
 // 214 registers, also one CTA per SM, left half as many dependent loads in flight: 96 LPs of 100 to
-// 1600 rows, 256 iterations with set-up and transfers, 42.2 ms, now 31.5 with the passes' sums taken
-// together and the CTA's sums a slot per thread.)
+// 1600 rows, 256 iterations with set-up and transfers, 42.2 ms, and 31.5 with 16 warps, the passes'
+// sums taken together and the CTA's sums a slot per thread.  No other kernel's CTA fits beside one any
+// more: two LPs of 30k rows solved beside 304 slots of 800 rows finish after 122 ms instead of 108 to
+// 115, the whole after 134 ms instead of 290.)
 constexpr int kBT = 512;
 // Threads whose chains of FP32 restart-norm sums a slot's results are defined by (see replay_*).
 constexpr int kChain = 256;

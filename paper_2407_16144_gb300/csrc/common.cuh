@@ -240,10 +240,10 @@ __host__ __device__ __forceinline__ void for_strided(int b, int e, int first, in
 }
 
 // ---------------------------------------------------------------------------------------------
-// FP64 comparisons on the integer pipe.  The FP64 pipe of this part takes about 19 clocks per warp
-// and SM for any instruction, a comparison, a maximum or an isfinite as long as a fused
-// multiply-add; the order of two doubles can be had from their bits.  All agree with the
-// floating-point comparison, NaN included.
+// FP64 comparisons on the integer pipe.  An FP64 instruction of a warp, a comparison, a maximum or an
+// isfinite as much as a fused multiply-add, holds its scheduler's part of the FP64 pipe for 64 clocks
+// (76 measured with 16 warps on an SM: 16 to 19 clocks per warp and SM); the order of two doubles can
+// be had from their bits.  All agree with the floating-point comparison, NaN included.
 
 __device__ __forceinline__ bool dbl_finite(double x) {
   return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
@@ -373,8 +373,9 @@ __device__ __forceinline__ double (*cta_red())[kMaxPartials] {
 // l / (32 / N).  While more than one slot is left, a lane keeps half of them and hands its partner
 // the other half, so 4 slots take 6 additions per lane instead of 20.  Each slot's additions are
 // those of warp_sum's tree (lanes 16, 8, 4, 2, 1 apart; an addition's operands may change places),
-// so the result has the same bits.  An FP64 addition takes 64 clocks whatever its mask, so a stage's
-// tail was mostly these trees: with it 75k entries in mixed precision 22.6 to 18.3 us an iteration.
+// so the result has the same bits.  An FP64 addition takes its scheduler 64 clocks whatever its mask,
+// so a stage's tail was mostly these trees: with it 75k entries in mixed precision 22.6 to 18.3 us an
+// iteration.
 template <int N, class T, class Add, class Xor>
 __device__ __forceinline__ T warp_reduce_slots(T (&v)[N], Add add, Xor from_xor) {
   static_assert(N == 1 || N == 2 || N == 4, "slots per reduction");
@@ -726,8 +727,9 @@ __device__ void dcol_finish(const DeferredCol &dc, const DcolPre &pre, double *o
 // entries with an L2 evict-first policy: where one iteration's bytes exceed L2 they stream through
 // once per product, and the policy leaves L2 to the gathered vectors and the reduction partials.
 // Where the problem fits L2 the plain loads (CP = 0) are kept: there the evict-first lines were
-// measured to cost re-reads; BF16 values keep them too (the hinted 8-byte loads measured slower).  The policy is created next to each load from an immediate, which
-// the compiler keeps a constant (a policy selected at run time measured slower).
+// measured to cost re-reads; BF16 values keep them too (the hinted 8-byte loads measured slower).
+// The policy is created next to each load from an immediate, which the compiler keeps a constant (a
+// policy selected at run time measured slower).
 __device__ __forceinline__ unsigned long long l2_evict_first() {
   unsigned long long p;
   asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
@@ -987,8 +989,9 @@ struct NoPrefetch {
 // Stage the products of the segment [seg_b, seg_e) (seg_b 4-aligned) in smem[0, ...): lane
 // handles 4-entry groups g = lane, lane + 32, ..., U at a time (more loads in flight per round,
 // more registers).  FP32 and ordered FP64 products are staged one by one.  Other FP64 products are
-// added up within their group of four, up to a row's end (a set bit of ends, see row_ends): smem[p] holds, where entry p
-// ends its row or its group, the sum of the row's entries in the group, and nothing elsewhere.
+// added up within their group of four, up to a row's end (a set bit of ends, see row_ends_clear):
+// smem[p] holds, where entry p ends its row or its group, the sum of the row's entries in the group,
+// and nothing elsewhere.
 template <typename VT, typename PT, int U, int CP, bool ORD, typename Src>
 __device__ __forceinline__ void stage_segment(const SideLayout &lay, const SideVals<VT> vals,
                                               const Src &src, PT *smem, int seg_b, int seg_e,

@@ -151,8 +151,9 @@ row_iter_mx(double *smem, const SideLayout &lay, const SideVals<double> v64,
     if (dcol)   // the deferred ordinary column stage's two sums (its packed slots)
       dcol_finish<col_df_slots<0>(), DFS == 1>(dc, pre, rc);
     if (threadIdx.x == 0) row_finalize(ctl, ic, r, t, k, n_ep, sigma, move, dcol, rc, !BOTH);
-    // (small LPs only, 75k entries 13.5 to 13.3 ms in 640 iterations: with 2.5M entries it measured
-    // 1% slower, in the FP64 kernels 2% slower on LPs beyond L2)
+    // (in the kernels of resident stages only, 75k entries 13.5 to 13.3 ms in 640 iterations: with
+    // 2.5M entries it measured 1% slower, in the FP64 kernels, which have one form for all sizes, 2%
+    // slower on LPs beyond L2)
     if (BOTH && threadIdx.x == blockDim.x - kWarp) halpern_weight(ctl, k);
   }
 }
@@ -161,7 +162,9 @@ row_iter_mx(double *smem, const SideLayout &lay, const SideVals<double> v64,
 // (MODE 2) takes both kinds of iteration.  Elsewhere the two are launched one after the other in
 // every iteration, which keeps the register footprint of the ordinary kernel small and its
 // residency high; a launch that returns at entry costs about 1.3 us.  75k entries, 640 iterations
-// with create and free: 16.2 to 14.3 ms (with the power iteration's unread norms left out).
+// with create and free: 16.2 to 14.3 ms (with the power iteration's unread norms left out).  BF16
+// values and double-float sums have no MODE 2 instantiations and keep the two launches at every size;
+// what one kernel would give them has not been measured.
 template <int RHO2, int MODE, int WALK, int DFS, int LP, int CP = 0>
 __global__ void __maxnreg__(mx_max_regs(MODE, WALK, DFS))
 k_row_iter_mx(SideLayout lay, SideVals<double> v64, SideVals<LowT<LP>> v32, WalkScratch wa,
@@ -316,8 +319,9 @@ __global__ void k_zero_f32(int n, float *x) {
 }  // namespace
 
 // The restart-mode kernel (MODE 1) of each stage is launched first and returns at entry unless
-// the stage needs it (both: one kernel, MODE 2, in their place); the ordinary kernel (MODE 0) follows, in the instantiation of the side's
-// walk (SideLayout::walk) and of the solve's restart-norm sums (IterConsts::df_sums).
+// the stage needs it (both: one kernel, MODE 2, in their place); the ordinary kernel (MODE 0)
+// follows, in the instantiation of the side's walk (SideLayout::walk) and of the solve's restart-norm
+// sums (IterConsts::df_sums).
 template <int V>
 using IC = std::integral_constant<int, V>;
 

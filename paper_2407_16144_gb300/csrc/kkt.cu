@@ -30,7 +30,9 @@ constexpr int kKktRowSlots = 3;            // the first three come from the row 
 constexpr int kKktFlag = 5;                // dout[5]: 1 if the CSR held an index out of range
 constexpr int kKktStage = 704;             // entries a warp stages at a time (22 per row of 32): a
                                            // multiple of 4
-constexpr int kKktRowCtas = 4;             // resident CTAs per SM of the row kernel (45 KB each)
+constexpr int kKktRowCtas = 4;             // resident CTAs per SM of the row kernel: 45 KB each, and 64
+                                           // registers a thread, under which it spills (76 bytes of
+                                           // stores, 52 of loads); fewer CTAs were not measured
 
 __device__ __forceinline__ double block_sum(double v, double *sh) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

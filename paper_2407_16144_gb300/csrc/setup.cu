@@ -102,7 +102,8 @@ __global__ void k_gather_csc(int nnz, const int *perm, const int *rows_of, const
 // instructions) run on packed rows, not in the one lane of a group that has the statistic (61 to 77
 // ms for the create below).  Not a reciprocal square root: on matrices of +-1 the factors lie on
 // the ties of the rounding to powers of two, where the last bit decides.  Create, 64 iterations and
-// free, with k_copy_rows: 30M entries 61.1 to 47.4 ms, 2.5M entries 11.4 to 10.0 ms.
+// free, with few lanes a row in k_copy_rows as well: 30M entries 61.1 to 47.4 ms, 2.5M entries 11.4
+// to 10.0 ms.
 constexpr int kStatLong = 32;
 
 template <int OP>
@@ -367,9 +368,10 @@ k_side_spmv_pw(SideLayout lay, SideVals<VT> vals, WalkScratch ws,
 // rows, a lane per row; the host reads back one summary and the arrays are written where they are
 // used.  (Planned on one host core, with the row pointers copied down and the arrays copied up, the
 // 10M columns and 1.75M rows of a 30M-entry flow LP took 42 of the 119 ms of create, 64 iterations
-// and free; the whole is 76 ms now.  250k columns and 100k rows: 14.5 to 13.3 ms.)  Three passes: k_plan_tiles makes every tile's long-row mask and
-// counts and each block's totals, k_plan_scan turns the totals into starts (one block; there is
-// one record per kPlanTiles tiles), k_plan_emit writes the arrays.
+// and free; planned here, the whole took 76 ms.  250k columns and 100k rows: 14.5 to 13.3 ms.)
+// Three passes: k_plan_tiles makes every tile's long-row mask and counts and each block's totals,
+// k_plan_scan turns the totals into starts (one block; there is one record per kPlanTiles tiles),
+// k_plan_emit writes the arrays.
 
 constexpr int kPlanTiles = 64;       // tiles of a block: 8 warps, 8 tiles each; a multiple of
                                      // kMaxTileMult, so that no tile group spans two blocks
