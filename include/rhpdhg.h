@@ -341,9 +341,9 @@ int rhpdhg_kernel_times(const rhpdhg_handle *h, double *ms_row, double *ms_col,
  * default stream) and the call synchronises it, so it must not be issued on a stream that is
  * being captured into a graph.  Scratch (n + 8200 doubles of device memory) is taken from the
  * process-wide cache of device buffers and goes back to it, so it stays allocated after the call
- * until it is evicted or rhpdhg_release_cached_memory is called.  Errors: RHPDHG_ERR_INVALID_ARG for host-memory, incomplete or
- * out-of-range input, RHPDHG_ERR_OOM / RHPDHG_ERR_CUDA on CUDA failures; each sets the message
- * of rhpdhg_last_error(NULL). */
+ * until it is evicted or rhpdhg_release_cached_memory is called.  Errors: RHPDHG_ERR_INVALID_ARG
+ * for host-memory, incomplete or out-of-range input, RHPDHG_ERR_OOM / RHPDHG_ERR_CUDA on CUDA
+ * failures; each sets the message of rhpdhg_last_error(NULL). */
 int rhpdhg_kkt_eval(const rhpdhg_problem *lp, const double *x, const double *y,
                     void *cuda_stream, double *out);
 
